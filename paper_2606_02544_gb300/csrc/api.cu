@@ -221,7 +221,7 @@ namespace simsd {
 RopeTable make_rope_table(double theta, int d) {
   RopeTable t{};
   for (int i = 0; i < d / 2 && i < 64; ++i) {
-    const double f = std::pow(theta, -2.0 * i / d);
+    const double f = std::pow(theta, -2.0 * i / d) / 3.14159265358979323846;
     const float hi = static_cast<float>(f);
     t.f[i] = make_float2(hi, static_cast<float>(f - static_cast<double>(hi)));
   }

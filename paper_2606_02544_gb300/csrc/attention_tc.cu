@@ -9,8 +9,8 @@
 // Eq. (1) visibility is evaluated on the fly from (section, tau), then the
 // cached prefix pages (read through the page table with TMA).  When the
 // inputs are not rotated yet (Sec. 3.1 RoPE copy), the softmax warps rotate
-// Q while moving it into TMEM and rotate the new keys in shared memory before
-// the first S is computed; cached keys are stored rotated.
+// Q and the new keys in shared memory before Q moves into TMEM and the first
+// S is computed (rope_tile.cuh); cached keys are stored rotated.
 //
 // Two CTAs share each SM (96 KB of shared memory, 256 TMEM columns and 192
 // threads apiece), so one CTA's set-up, first loads and epilogue overlap the
@@ -44,6 +44,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "ptx.cuh"
+#include "rope_tile.cuh"
 
 // Scratch of simsd_verify_attention_noalloc: the split partials live in this
 // file-scope array instead of caller memory.  Every device that loads the
@@ -115,6 +116,7 @@ struct alignas(1024) Smem {
   int seq_bad;
   int b_sel, n_sel;
   int32_t tau[64];
+  int32_t pos[64];  // kRope: RoPE positions of the slots
   uint8_t sect[64];
   int32_t pages[kPageCache];
 };
@@ -136,8 +138,9 @@ __device__ __forceinline__ uint4 ld_sw128_chunk(const uint8_t* half, int r, int 
 
 // kFuse: the prefix splits of a unit form a cluster and merge their partials
 // in shared memory (a separate instantiation, so that the unclustered kernel
-// carries no cluster barriers).
-template <bool kFuse>
+// carries no cluster barriers).  kRope: queries and new keys arrive unrotated
+// (also a separate instantiation: the plain one carries none of that code).
+template <bool kFuse, bool kRope>
 __global__ void __maxnreg__(kMaxRegs)
     attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kn,
                         const __grid_constant__ CUtensorMap tm_vn, const __grid_constant__ CUtensorMap tm_kc,
@@ -325,6 +328,7 @@ __global__ void __maxnreg__(kMaxRegs)
   for (int i = tid; i < p.S; i += kThreads) {
     sm.tau[i] = p.tau[static_cast<size_t>(b) * p.S + i];
     sm.sect[i] = p.section[static_cast<size_t>(b) * p.S + i];
+    if (kRope) sm.pos[i] = p.rope_pos[static_cast<size_t>(b) * p.S + i];
   }
   const bool n_bad = n < 0 || static_cast<long long>(n) > static_cast<long long>(p.max_pages) * p.page_size;
   if (n_bad) {
@@ -479,34 +483,38 @@ __global__ void __maxnreg__(kMaxRegs)
 
     // ---- Q: shared memory (ring slot 0) -> TMEM columns [0, 64)
     if (ntiles > 0) {
-      const int pos = p.rope_pos ? p.rope_pos[static_cast<size_t>(b) * p.S + (s < p.S ? s : 0)] : 0;
       ok = mbar_wait_warp(smem_u32(&sm.bar_k[0]), 0, abort_flag, p.wait_ns);
-      if (ok && p.rope_pos) {
-        // rotate this row's query at its slot's position on the way
-        const uint8_t* h0 = sm.ring[0];
-        const uint8_t* h1 = sm.ring[0] + 2 * kHalfBytes;
-        uint32_t q0r[32], q1r[32];
+      if (kRope) {
+        // rotate this unit's queries and, in the split that holds them (its
+        // first tile, ring item 1), the new keys at their slots' positions
+        constexpr int st1 = 1 % kStages;
+        const bool keys_here = t0 == 0;
+        if (ok && keys_here) ok = mbar_wait_warp(smem_u32(&sm.bar_k[st1]), 0, abort_flag, p.wait_ns);
+        if (ok) {
+          const int q4 = tid % kRopeThreadsPerSlot;
+          float2 f[4];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const uint4 va = ld_sw128_chunk(h0, row, c), vb = ld_sw128_chunk(h1, row, c);
-          const uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            float x0 = __uint_as_float(wa[w] << 16), x1 = __uint_as_float(wa[w] & 0xffff0000u);
-            float y0 = __uint_as_float(wb[w] << 16), y1 = __uint_as_float(wb[w] & 0xffff0000u);
-            float sn, cs;
-            rope_sincos(pos, p.rope.f[8 * c + 2 * w], &sn, &cs);
-            rope_pair(x0, y0, sn, cs);
-            rope_sincos(pos, p.rope.f[8 * c + 2 * w + 1], &sn, &cs);
-            rope_pair(x1, y1, sn, cs);
-            q0r[4 * c + w] = pack_bf16x2(x0, x1);
-            q1r[4 * c + w] = pack_bf16x2(y0, y1);
+          for (int e = 0; e < 4; ++e) f[e] = p.rope.f[4 * q4 + e];
+          const int s0 = rblk * p.s_blk, s1 = min(p.S, s0 + p.s_blk);  // the slots of this block's query rows
+          const int lo = keys_here ? 0 : s0, hi = keys_here ? p.S : s1;
+#pragma unroll 1
+          for (int t = lo + tid / kRopeThreadsPerSlot; t < hi; t += 128 / kRopeThreadsPerSlot) {
+            float sn[4], cs[4];
+            rope_angles4(sm.pos[t], f, sn, cs);
+            if (t >= s0 && t < s1) {
+#pragma unroll 2
+              for (int j = 0; j < p.g; ++j)
+                rope_rotate4(sm.ring[0], sm.ring[0] + 2 * kHalfBytes, (t - s0) * p.g + j, q4, sn, cs);
+            }
+            if (keys_here) rope_rotate4(sm.ring[st1], sm.ring[st1] + kHalfBytes, t, q4, sn, cs);
           }
+          // read next by the tensor core (keys) and overwritten by TMA (the
+          // queries' slot)
+          fence_proxy_async_smem();
         }
-        tmem_st32(lane_tmem + kColQ, q0r);
-        tmem_st32(lane_tmem + kColQ + 32, q1r);
-        tmem_wait_st();
-      } else if (ok) {
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+      }
+      if (ok) {
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
           const uint8_t* half = sm.ring[0] + h * 2 * kHalfBytes;
@@ -522,39 +530,6 @@ __global__ void __maxnreg__(kMaxRegs)
           tmem_st32(lane_tmem + kColQ + 32 * h, qr);
         }
         tmem_wait_st();
-      }
-      if (ok && p.rope_pos && t0 == 0) {
-        // the new keys (ring item 1, the unit's first tile) are rotated in
-        // place before the first S = Q K^T reads them
-        constexpr int st1 = 1 % kStages;
-        ok = mbar_wait_warp(smem_u32(&sm.bar_k[st1]), 0, abort_flag, p.wait_ns);
-        if (ok) {
-          uint8_t* h0 = sm.ring[st1];
-          uint8_t* h1 = sm.ring[st1] + kHalfBytes;
-          for (int task = tid; task < p.S * 8; task += 128) {
-            const int r = task >> 3, c = task & 7;
-            const int pos = p.rope_pos[static_cast<size_t>(b) * p.S + r];
-            uint4* pa = reinterpret_cast<uint4*>(h0 + r * 128 + ((c ^ (r & 7)) << 4));
-            uint4* pb = reinterpret_cast<uint4*>(h1 + r * 128 + ((c ^ (r & 7)) << 4));
-            const uint4 va = *pa, vb = *pb;
-            uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-              float x0 = __uint_as_float(wa[w] << 16), x1 = __uint_as_float(wa[w] & 0xffff0000u);
-              float y0 = __uint_as_float(wb[w] << 16), y1 = __uint_as_float(wb[w] & 0xffff0000u);
-              float sn, cs;
-              rope_sincos(pos, p.rope.f[8 * c + 2 * w], &sn, &cs);
-              rope_pair(x0, y0, sn, cs);
-              rope_sincos(pos, p.rope.f[8 * c + 2 * w + 1], &sn, &cs);
-              rope_pair(x1, y1, sn, cs);
-              wa[w] = pack_bf16x2(x0, x1);
-              wb[w] = pack_bf16x2(y0, y1);
-            }
-            *pa = make_uint4(wa[0], wa[1], wa[2], wa[3]);
-            *pb = make_uint4(wb[0], wb[1], wb[2], wb[3]);
-          }
-          fence_proxy_async_smem();
-        }
       }
       tc_fence_before();
       asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -945,7 +920,8 @@ cudaError_t ensure_smem_attr() {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(mu);
   if (done[dev]) return cudaSuccess;
-  for (auto kern : {attention_tc_kernel<false>, attention_tc_kernel<true>}) {
+  for (auto kern : {attention_tc_kernel<false, false>, attention_tc_kernel<false, true>,
+                    attention_tc_kernel<true, false>, attention_tc_kernel<true, true>}) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes()));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -1121,11 +1097,10 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, const AttnTcPlan& pl, Encod
     if (e != cudaSuccess) return e;
   }
   const long long grid = static_cast<long long>(a.Bt) * pl.nsplit * a.Hkv * pl.rb;
-  cudaError_t e = pl.fuse ? launch_overlapped(attention_tc_kernel<true>, dim3(static_cast<unsigned>(grid)),
-                                               dim3(kThreads), smem_bytes(), stream,
-                                               static_cast<unsigned>(pl.nsplit), tq, tkn, tvn, tkc, tvc, p)
-                          : launch_overlapped(attention_tc_kernel<false>, dim3(static_cast<unsigned>(grid)),
-                                              dim3(kThreads), smem_bytes(), stream, 1u, tq, tkn, tvn, tkc, tvc, p);
+  auto kern = a.rope_pos ? (pl.fuse ? attention_tc_kernel<true, true> : attention_tc_kernel<false, true>)
+                         : (pl.fuse ? attention_tc_kernel<true, false> : attention_tc_kernel<false, false>);
+  cudaError_t e = launch_overlapped(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreads), smem_bytes(), stream,
+                                    pl.fuse ? static_cast<unsigned>(pl.nsplit) : 1u, tq, tkn, tvn, tkc, tvc, p);
   if (e != cudaSuccess || pl.nsplit == 1 || pl.fuse) return e;
   const long long warps = static_cast<long long>(a.Bt) * a.Hkv * pl.rb * pl.rows_blk;
   return launch_combine(p, warps, pl.num_sms, stream);

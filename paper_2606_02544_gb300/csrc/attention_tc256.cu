@@ -59,6 +59,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "ptx.cuh"
+#include "rope_tile.cuh"
 
 namespace simsd {
 namespace {
@@ -133,31 +134,6 @@ static_assert(smem_bytes() <= 232448, "one CTA per SM");
 __device__ __forceinline__ void signal_abort(Smem256& sm, int32_t* err_word) {
   raise_error(err_word, SIMSD_EW_TIMEOUT);
   *reinterpret_cast<volatile int*>(&sm.abort_flag) = 1;
-}
-
-// Row r of a 128-byte-swizzled tile: 16-byte chunk c sits at chunk c ^ (r & 7).
-__device__ __forceinline__ uint4* sw128_chunk(uint8_t* half, int r, int c) {
-  return reinterpret_cast<uint4*>(half + r * 128 + ((c ^ (r & 7)) << 4));
-}
-
-// Rotates the pairs (x_i, x_{i+64}) held in chunk c of two d-halves in place.
-__device__ __forceinline__ void rope_chunk_pair(uint4* pa, uint4* pb, int pos, int c, const RopeTable& rope) {
-  const uint4 va = *pa, vb = *pb;
-  uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
-#pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    float x0 = __uint_as_float(wa[w] << 16), x1 = __uint_as_float(wa[w] & 0xffff0000u);
-    float y0 = __uint_as_float(wb[w] << 16), y1 = __uint_as_float(wb[w] & 0xffff0000u);
-    float sn, cs;
-    rope_sincos(pos, rope.f[8 * c + 2 * w], &sn, &cs);
-    rope_pair(x0, y0, sn, cs);
-    rope_sincos(pos, rope.f[8 * c + 2 * w + 1], &sn, &cs);
-    rope_pair(x1, y1, sn, cs);
-    wa[w] = pack_bf16x2(x0, x1);
-    wb[w] = pack_bf16x2(y0, y1);
-  }
-  *pa = make_uint4(wa[0], wa[1], wa[2], wa[3]);
-  *pb = make_uint4(wb[0], wb[1], wb[2], wb[3]);
 }
 
 // Tiles of a unit of a sequence with prefix length n: ceil(n / 64) + 1 (tile
@@ -344,6 +320,9 @@ __device__ __forceinline__ int4* streamk_records(const Tc256Params& p) {
   return reinterpret_cast<int4*>(p.ws + partial_entries(p) * kRows * (kD + 2));
 }
 
+// kRope: queries and new keys arrive unrotated (an instantiation of its own:
+// the plain kernel carries none of that code).
+template <bool kRope>
 __global__ void __launch_bounds__(kThreads, 1)
     attention_tc256_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kn,
                            const __grid_constant__ CUtensorMap tm_vn, const __grid_constant__ CUtensorMap tm_kc,
@@ -414,11 +393,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = sm.tmem_base;
 
   // Register split (setmaxnreg, per warpgroup): the two softmax warpgroups
-  // take 200 registers a thread, the two control warpgroups give theirs
-  // down to 56 (2 x 128 x 200 + 2 x 128 x 56 = 65,536, the 512 x 128 the
-  // block is launched with).
+  // take 192 registers a thread, the two control warpgroups give theirs
+  // down to 64 (2 x 128 x 192 + 2 x 128 x 64 = 65,536, the 512 x 128 the
+  // block is launched with; at 56 the control warps spilled 28 bytes).
   if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     if (warp == kWarpProducer || warp == kWarpProducerV) {
       // ----------------------------------------------------------- producers
       // warp 8 loads Q and the K half of every tile, warp 11 the V half; each
@@ -551,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t g0 = g, g_end = g + u.tiles;
           if (is_s) {
             // Q landed (rotated by the softmax warps when RoPE is applied here)
-            ok = mbar_wait(smem_u32(p.rope_pos ? &sm.bar_qr : &sm.bar_q), (jq - 1) & 1, abort_flag, p.wait_ns);
+            ok = mbar_wait(smem_u32(kRope ? &sm.bar_qr : &sm.bar_q), (jq - 1) & 1, abort_flag, p.wait_ns);
             for (uint32_t gg = g0; ok && gg < g_end; ++gg) {
               // S_X(t) needs K(t) and the completion of PV_X(t - 2), which read
               // the P held in the same S buffer
@@ -606,7 +585,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
     // -------------------------------------------------------------- softmax
     const int x = warp >> 2;          // row block
     const int row = tid & (kRows - 1);  // TMEM lane / query row of the block
@@ -657,27 +636,34 @@ __global__ void __launch_bounds__(kThreads, 1)
       float m_ref = -INFINITY, l_sum = 0.f;
       if (u.tiles > 0) {
         ++jq;
-        if (p.rope_pos) {
+        if (kRope) {
           // Q of both blocks and, in range 0, the new keys (its first tile)
-          // are rotated in shared memory before the first S reads them
-          const int pos = p.rope_pos[static_cast<size_t>(u.b) * p.S + (row_exists ? s : 0)];
-          if (ok) ok = mbar_wait_warp(smem_u32(&sm.bar_q), (jq - 1) & 1, abort_flag, p.wait_ns);
-          if (ok) {
-            uint8_t* h0 = sm.q[x];
-            uint8_t* h1 = sm.q[x] + kQHalfBytes;
-#pragma unroll 1
-            for (int c = 0; c < 8; ++c) rope_chunk_pair(sw128_chunk(h0, row, c), sw128_chunk(h1, row, c), pos, c, p.rope);
-          }
+          // are rotated in shared memory before the first S reads them: 16
+          // threads a slot, 16 slots at a time, the next slot's position
+          // loaded ahead
+          constexpr int kSlots = kSoftmaxThreads / kRopeThreadsPerSlot;
+          const int q4 = tid % kRopeThreadsPerSlot;
+          int t = tid / kRopeThreadsPerSlot;
+          const int32_t* pos_b = p.rope_pos + static_cast<size_t>(u.b) * p.S;
+          int pos = t < p.S ? pos_b[t] : 0;
+          float2 f[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) f[e] = p.rope.f[4 * q4 + e];
           const int st0 = g % kStages;
+          if (ok) ok = mbar_wait_warp(smem_u32(&sm.bar_q), (jq - 1) & 1, abort_flag, p.wait_ns);
           if (ok && u.t0 == 0) ok = mbar_wait_warp(smem_u32(&sm.bar_k[st0]), (g / kStages) & 1, abort_flag, p.wait_ns);
-          if (ok && u.t0 == 0) {
-            uint8_t* h0 = sm.ring[st0];
-            uint8_t* h1 = sm.ring[st0] + kHalfBytes;
-            for (int task = tid; task < p.S * 8; task += kSoftmaxThreads) {
-              const int r = task >> 3, c = task & 7;
-              const int kpos = p.rope_pos[static_cast<size_t>(u.b) * p.S + r];
-              rope_chunk_pair(sw128_chunk(h0, r, c), sw128_chunk(h1, r, c), kpos, c, p.rope);
-            }
+#pragma unroll 1
+          for (; ok && t < p.S; t += kSlots) {
+            const int pos_t = pos;
+            if (t + kSlots < p.S) pos = pos_b[t + kSlots];
+            float sn[4], cs[4];
+            rope_angles4(pos_t, f, sn, cs);
+            const int xb = t >= p.s_blk ? 1 : 0;
+            uint8_t* h0 = sm.q[xb];
+#pragma unroll 2
+            for (int i = 0; i < p.g; ++i)
+              rope_rotate4(h0, h0 + kQHalfBytes, (t - xb * p.s_blk) * p.g + i, q4, sn, cs);
+            if (u.t0 == 0) rope_rotate4(sm.ring[st0], sm.ring[st0] + kHalfBytes, t, q4, sn, cs);
           }
           fence_proxy_async_smem();
           asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -1161,16 +1147,18 @@ cudaError_t launch_attention_tc256(const AttnTcArgs& a, const AttnTcPlan& pl, En
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(mu);
     if (!done[dev]) {
-      e = cudaFuncSetAttribute(attention_tc256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(smem_bytes()));
-      if (e != cudaSuccess) return e;
+      for (auto k : {attention_tc256_kernel<false>, attention_tc256_kernel<true>}) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes()));
+        if (e != cudaSuccess) return e;
+      }
       done[dev] = true;
     }
   }
   const int grid = pl.streamk ? pl.num_sms : std::min(p.items, pl.num_sms);
   p.ctas = grid;
-  cudaError_t e = launch_overlapped(attention_tc256_kernel, dim3(static_cast<unsigned>(grid)), dim3(kThreads),
-                                    smem_bytes(), stream, 1u, tq, tkn, tvn, tkc, tvc, p);
+  cudaError_t e = launch_overlapped(a.rope_pos ? attention_tc256_kernel<true> : attention_tc256_kernel<false>,
+                                    dim3(static_cast<unsigned>(grid)), dim3(kThreads), smem_bytes(), stream, 1u, tq,
+                                    tkn, tvn, tkc, tvc, p);
   if (e != cudaSuccess) return e;
   if (pl.streamk)
     return grid > 1 ? launch_overlapped(streamk_combine_kernel, dim3(static_cast<unsigned>(grid - 1), 2u, kRows / 16),

@@ -69,27 +69,21 @@ inline cudaError_t launch_overlapped(void (*kern)(KArgs...), dim3 grid, dim3 blo
 
 // ---- rotary position embedding (Su et al., RoFormer), rotate-half layout:
 // for i < d/2 the pair (x_i, x_{i+d/2}) turns by the angle pos * theta^(-2i/d).
-// The per-pair frequencies theta^(-2i/d) come in a RopeTable (kernels.h).
+// The per-pair frequencies theta^(-2i/d) / pi come in a RopeTable (kernels.h).
 
-// sin and cos of pos * f for 0 <= pos < 2^24.  The product is kept in
-// float-float (the rounding error of p * hi comes back exactly from an FMA)
-// and reduced to [-pi, pi] by Cody-Waite subtraction of k * 2pi, with 2pi
-// split into three floats of which the first has 8 significant bits, so the
-// first subtraction is exact; the reduced angle is good to ~2e-7 rad up to
-// pos = 2^20.
+// sin and cos of pi * pos * f for 0 <= pos < 2^24.  Angles are counted in
+// half turns: the product is kept in float-float (the rounding error of p * hi
+// comes back exactly from an FMA) and whole turns are subtracted exactly (an
+// even integer from a float of at least its last place), so only r + b and
+// the sine and cosine themselves round.  sincospi needs no further range
+// reduction: sincosf spends most of its instructions on one, with a branch to
+// local memory for huge arguments that never come here.
 __device__ __forceinline__ void rope_sincos(int pos, float2 f, float* sn, float* cs) {
-  constexpr float kTwoPiA = 6.28125f;
-  constexpr float kTwoPiB = 1.9353071693331003e-03f;
-  constexpr float kTwoPiC = 1.0253131677018246e-11f;
-  constexpr float kInvTwoPi = 0.15915493667125702f;
   const float p = static_cast<float>(pos);
   const float a = p * f.x;
   const float b = fmaf(p, f.y, fmaf(p, f.x, -a));
-  const float k = rintf(a * kInvTwoPi);
-  float r = fmaf(-k, kTwoPiA, a);
-  r = fmaf(-k, kTwoPiB, r);
-  r = fmaf(-k, kTwoPiC, r);
-  sincosf(r + b, sn, cs);
+  const float r = fmaf(-2.0f, rintf(0.5f * a), a);
+  sincospif(r + b, sn, cs);
 }
 
 // Rotates one pair in place.

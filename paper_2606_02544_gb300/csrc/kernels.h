@@ -8,8 +8,9 @@
 
 namespace simsd {
 
-// Rotary embedding frequencies theta^(-2i/d), i < d/2 <= 64, each as an
-// unevaluated sum f.x + f.y of two floats (rounded from double).
+// Rotary embedding frequencies in half turns per position, theta^(-2i/d) / pi,
+// i < d/2 <= 64, each as an unevaluated sum f.x + f.y of two floats (rounded
+// from double).
 struct RopeTable {
   float2 f[64];
 };
