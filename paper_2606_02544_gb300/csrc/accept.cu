@@ -4,9 +4,9 @@
 //
 // One thread-block cluster per sequence.  The CTAs of a cluster split the
 // sequence's [gamma+1][vocab] block into contiguous spans; each thread
-// streams 16-byte loads (8 or 16 in flight), keeps a running (value, index) per
-// row with plain float compares, and folds it into a 64-bit key per row in
-// shared memory when its row changes.
+// streams 16-byte loads (8 or 16 in flight), whatever the rows' alignment,
+// keeps a running (value, index) per row with plain float compares, and folds
+// it into a 64-bit key per row in shared memory when its row changes.
 // Each CTA then writes its keys into CTA 0's shared memory (distributed
 // shared memory) and arrives on an mbarrier there, and exits; CTA 0 waits for
 // the CL arrivals, takes the maximum per row and walks the draft order.  No
@@ -69,20 +69,30 @@ struct RowBest {
     v = gt ? x : v;
     i = gt ? e : i;
   }
+  // four values from index e on
+  __device__ __forceinline__ void see4(const float4& x, uint32_t e) {
+    if (isnan(x.x) | isnan(x.y) | isnan(x.z) | isnan(x.w)) {
+      if (nan_i == 0xFFFFFFFFu) nan_i = isnan(x.x) ? e : isnan(x.y) ? e + 1 : isnan(x.z) ? e + 2 : e + 3;
+    }
+    see(x.x, e);
+    see(x.y, e + 1);
+    see(x.z, e + 2);
+    see(x.w, e + 3);
+  }
   __device__ __forceinline__ unsigned long long key() const {
     return nan_i != 0xFFFFFFFFu ? argmax_key(__int_as_float(0x7fc00000), nan_i) : argmax_key(v, i);
   }
 };
 
-// Span c of CL equal spans of one sequence's [rows][vocab] block (in 16-byte
-// units when rows are 16-byte aligned): each thread streams its elements
-// and folds a running (value, index) per row into best[row] (shared memory,
-// 64-bit keys, atomicMax) when its row changes.
+// Span c of CL equal spans of one sequence's [rows][vocab] block, whose rows
+// start on 16-byte boundaries, in units of 16 bytes: each thread streams its
+// units and folds a running (value, index) per row into best[row] (shared
+// memory, 64-bit keys, atomicMax) when its row changes.
 template <int UNROLL>
-__device__ __forceinline__ void scan_span(const float* __restrict__ base, int rows, int vocab, int vec4, int c, int CL,
-                                          unsigned long long* best) {
+__device__ __forceinline__ void scan_span_vec(const float* __restrict__ base, int rows, int vocab, int c, int CL,
+                                              unsigned long long* best) {
   const int tid = threadIdx.x;
-  const int W = vec4 ? (vocab >> 2) : vocab;   // units per row
+  const int W = vocab >> 2;  // units per row
   const long long F = static_cast<long long>(rows) * W;
   const long long per = (F + CL - 1) / CL;
   const long long f0 = min(F, c * per), f1 = min(F, f0 + per);
@@ -91,51 +101,25 @@ __device__ __forceinline__ void scan_span(const float* __restrict__ base, int ro
   int col = static_cast<int>(f - static_cast<long long>(row) * W);
   int cur = row;
   RowBest rb;
-  rb.reset(vec4 ? 4u * col : static_cast<uint32_t>(col));
+  rb.reset(4u * col);
   constexpr int kStride = kAcceptThreads;
-  if (vec4) {
-    const float4* b4 = reinterpret_cast<const float4*>(base);
-    for (; f < f1; f += static_cast<long long>(kStride) * UNROLL) {
-      float4 v[UNROLL];
+  const float4* b4 = reinterpret_cast<const float4*>(base);
+  for (; f < f1; f += static_cast<long long>(kStride) * UNROLL) {
+    float4 v[UNROLL];
 #pragma unroll
-      for (int u = 0; u < UNROLL; ++u) {
-        const long long fu = f + static_cast<long long>(u) * kStride;
-        if (fu < f1) v[u] = ld_stream_f4(reinterpret_cast<const float*>(b4 + fu));
-      }
-#pragma unroll
-      for (int u = 0; u < UNROLL; ++u) {
-        if (f + static_cast<long long>(u) * kStride >= f1) break;
-        if (row != cur) {
-          atomicMax(&best[cur], rb.key());
-          cur = row;
-          rb.reset(4u * col);
-        }
-        const uint32_t e = 4u * static_cast<uint32_t>(col);
-        if (isnan(v[u].x) | isnan(v[u].y) | isnan(v[u].z) | isnan(v[u].w)) {
-          if (rb.nan_i == 0xFFFFFFFFu)
-            rb.nan_i = isnan(v[u].x) ? e : isnan(v[u].y) ? e + 1 : isnan(v[u].z) ? e + 2 : e + 3;
-        }
-        rb.see(v[u].x, e);
-        rb.see(v[u].y, e + 1);
-        rb.see(v[u].z, e + 2);
-        rb.see(v[u].w, e + 3);
-        col += kStride;
-        if (col >= W) {
-          row += col / W;
-          col %= W;
-        }
-      }
+    for (int u = 0; u < UNROLL; ++u) {
+      const long long fu = f + static_cast<long long>(u) * kStride;
+      if (fu < f1) v[u] = ld_stream_f4(reinterpret_cast<const float*>(b4 + fu));
     }
-  } else {
-    for (; f < f1; f += kStride) {
-      const float x = __ldg(base + f);
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      if (f + static_cast<long long>(u) * kStride >= f1) break;
       if (row != cur) {
         atomicMax(&best[cur], rb.key());
         cur = row;
-        rb.reset(col);
+        rb.reset(4u * col);
       }
-      if (isnan(x) && rb.nan_i == 0xFFFFFFFFu) rb.nan_i = col;
-      rb.see(x, static_cast<uint32_t>(col));
+      rb.see4(v[u], 4u * static_cast<uint32_t>(col));
       col += kStride;
       if (col >= W) {
         row += col / W;
@@ -144,6 +128,102 @@ __device__ __forceinline__ void scan_span(const float* __restrict__ base, int ro
     }
   }
   if (f0 + tid < f1) atomicMax(&best[cur], rb.key());
+}
+
+// The same when rows start off the 16-byte grid (a vocabulary that is no
+// multiple of 4, or a base that is not 16-byte aligned).  Units of 16 bytes
+// are laid over the block as a whole, so a unit may hold the end of one row
+// and the start of the next (its values are then seen one by one), and the
+// first and the last unit may reach past the block (their values inside it
+// are loaded one by one).  Against one 4-byte load at a time, which this
+// replaced, 16 sequences of 9 rows of 50001 logits: 20.0 -> 10.9 us (the
+// host's calls by then); 64 sequences 69.7 -> 27.7 us.
+template <int UNROLL>
+__device__ __forceinline__ void scan_span_any(const float* __restrict__ base, int rows, int vocab, int c, int CL,
+                                              unsigned long long* best) {
+  const int tid = threadIdx.x;
+  const int h = static_cast<int>((reinterpret_cast<uintptr_t>(base) & 15u) >> 2);  // values of unit 0 before the block
+  const long long E = static_cast<long long>(rows) * vocab;
+  const long long F = (h + E + 3) >> 2;
+  const long long per = (F + CL - 1) / CL;
+  const long long f0 = min(F, c * per), f1 = min(F, f0 + per);
+  const float4* b4 = reinterpret_cast<const float4*>(base - h);
+  long long f = f0 + tid;
+  // the unit's first value: value e = 4 f - h of the block, column col of
+  // its row (col = -h < 0 in unit 0)
+  int row = 0, col = -h;
+  if (f > 0) {
+    row = static_cast<int>((4 * f - h) / vocab);
+    col = static_cast<int>(4 * f - h - static_cast<long long>(row) * vocab);
+  }
+  int cur = row;
+  RowBest rb;
+  rb.reset(static_cast<uint32_t>(max(col, 0)));
+  constexpr int kStride = kAcceptThreads;
+  for (; f < f1; f += static_cast<long long>(kStride) * UNROLL) {
+    float4 v[UNROLL];
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      const long long fu = f + static_cast<long long>(u) * kStride;
+      if (fu < f1) {
+        const long long e = 4 * fu - h;
+        if (e >= 0 && e + 3 < E) {
+          v[u] = ld_stream_f4(reinterpret_cast<const float*>(b4 + fu));
+        } else {
+          v[u].x = e >= 0 ? __ldg(base + e) : -INFINITY;  // (e < E: the unit holds a value)
+          v[u].y = e + 1 >= 0 && e + 1 < E ? __ldg(base + e + 1) : -INFINITY;
+          v[u].z = e + 2 >= 0 && e + 2 < E ? __ldg(base + e + 2) : -INFINITY;
+          v[u].w = e + 3 < E ? __ldg(base + e + 3) : -INFINITY;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      if (f + static_cast<long long>(u) * kStride >= f1) break;
+      if (row != cur) {
+        atomicMax(&best[cur], rb.key());
+        cur = row;
+        rb.reset(static_cast<uint32_t>(max(col, 0)));
+      }
+      if (col >= 0 && col + 3 < vocab) {
+        rb.see4(v[u], static_cast<uint32_t>(col));
+      } else {
+        const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+        int r = row, k = col;
+#pragma unroll
+        for (int q = 0; q < 4; ++q, ++k) {
+          if (k == vocab) {
+            k = 0;
+            ++r;
+          }
+          if (k < 0 || r >= rows) continue;  // past the block
+          if (r != cur) {
+            atomicMax(&best[cur], rb.key());
+            cur = r;
+            rb.reset(static_cast<uint32_t>(k));
+          }
+          if (isnan(x[q]) && rb.nan_i == 0xFFFFFFFFu) rb.nan_i = static_cast<uint32_t>(k);
+          rb.see(x[q], static_cast<uint32_t>(k));
+        }
+      }
+      col += 4 * kStride;
+      if (col >= vocab) {
+        row += col / vocab;
+        col %= vocab;
+      }
+    }
+  }
+  if (f0 + tid < f1) atomicMax(&best[cur], rb.key());
+}
+
+// VEC: rows start on 16-byte boundaries.
+template <int UNROLL, bool VEC>
+__device__ __forceinline__ void scan_span(const float* __restrict__ base, int rows, int vocab, int c, int CL,
+                                          unsigned long long* best) {
+  if constexpr (VEC)
+    scan_span_vec<UNROLL>(base, rows, vocab, c, CL, best);
+  else
+    scan_span_any<UNROLL>(base, rows, vocab, c, CL, best);
 }
 
 // One warp of sequence b, after am[r] (shared memory) holds the argmax of
@@ -174,13 +254,12 @@ __device__ __forceinline__ void walk_drafts(const int* am, int dr_lane, int b, i
 
 // UNROLL 16-byte loads are in flight per thread: 8 in general, 16 when the
 // grid leaves SMs idle (then each CTA has the SM to itself).
-template <int UNROLL>
-__global__ void __launch_bounds__(kAcceptThreads) accept_kernel(const float* __restrict__ logits,
-                                                                const int32_t* __restrict__ draft, int gamma,
-                                                                int vocab, int vec4, int32_t* __restrict__ accepted_len,
-                                                                int32_t* __restrict__ out_tokens,
-                                                                int32_t* __restrict__ row_argmax, int32_t* err_word,
-                                                                uint32_t extra_arrivals, unsigned long long wait_ns) {
+template <int UNROLL, bool VEC>
+__global__ void __launch_bounds__(kAcceptThreads, UNROLL == 8 ? 2 : 1)
+    accept_kernel(const float* __restrict__ logits, const int32_t* __restrict__ draft, int gamma, int vocab,
+                  int32_t* __restrict__ accepted_len, int32_t* __restrict__ out_tokens,
+                  int32_t* __restrict__ row_argmax, int32_t* err_word, uint32_t extra_arrivals,
+                  unsigned long long wait_ns) {
   __shared__ unsigned long long best[kMaxRows];
   __shared__ unsigned long long gath[kMaxCluster][kMaxRows];  // CTA 0: every CTA's keys
   __shared__ __align__(8) unsigned long long gbar;              // CTA 0: one arrival per CTA
@@ -206,7 +285,7 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(const float* __r
 
   // This CTA owns one contiguous span of the sequence's [rows][vocab] block
   // (in 16-byte units when rows are 16-byte aligned).
-  scan_span<UNROLL>(logits + static_cast<size_t>(b) * rows * vocab, rows, vocab, vec4, c, CL, best);
+  scan_span<UNROLL, VEC>(logits + static_cast<size_t>(b) * rows * vocab, rows, vocab, c, CL, best);
   // the next kernel may be scheduled once the stream of logits is done
   // (earlier, its waiting CTAs would sit beside this one's)
   pdl_launch_next();
@@ -245,9 +324,10 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(const float* __r
 // per row and walks the drafts.  The merge launch is let in as soon as this
 // grid has started, so that its launch latency hides behind the streaming
 // (its blocks, one per sequence, only wait for this grid to complete).
-__global__ void __launch_bounds__(kAcceptThreads) accept_part_kernel(const float* __restrict__ logits, int gamma,
-                                                                     int vocab, int vec4, int parts,
-                                                                     unsigned long long* __restrict__ keys) {
+template <bool VEC>
+__global__ void __launch_bounds__(kAcceptThreads, 2)
+    accept_part_kernel(const float* __restrict__ logits, int gamma, int vocab, int parts,
+                       unsigned long long* __restrict__ keys) {
   __shared__ unsigned long long best[kMaxRows];
   const int b = blockIdx.x / parts, c = blockIdx.x - b * parts;
   const int rows = gamma + 1;
@@ -255,7 +335,7 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_part_kernel(const float
   pdl_wait();
   pdl_launch_next();
   __syncthreads();
-  scan_span<8>(logits + static_cast<size_t>(b) * rows * vocab, rows, vocab, vec4, c, parts, best);
+  scan_span<8, VEC>(logits + static_cast<size_t>(b) * rows * vocab, rows, vocab, c, parts, best);
   __syncthreads();
   for (int r = threadIdx.x; r < rows; r += kAcceptThreads)
     keys[(static_cast<size_t>(b) * rows + r) * parts + c] = best[r];
@@ -337,8 +417,11 @@ cudaError_t cluster_capacity(const ClusterCapacity** out) {
   std::lock_guard<std::mutex> lk(mu);
   ClusterCapacity& c = cap[dev];
   if (!c.ready) {
-    e = cudaFuncSetAttribute(accept_kernel<UNROLL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
+    // (both layouts' kernels have the same register and shared-memory bounds)
+    for (auto kern : {accept_kernel<UNROLL, true>, accept_kernel<UNROLL, false>}) {
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
     for (int cl = 1; cl <= kMaxCluster; ++cl) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(static_cast<unsigned>(cl));
@@ -351,7 +434,7 @@ cudaError_t cluster_capacity(const ClusterCapacity** out) {
       cfg.attrs = attr;
       cfg.numAttrs = 1;
       int n = 0;
-      e = cudaOccupancyMaxActiveClusters(&n, accept_kernel<UNROLL>, &cfg);
+      e = cudaOccupancyMaxActiveClusters(&n, accept_kernel<UNROLL, true>, &cfg);
       if (e != cudaSuccess) return e;
       c.resident[cl] = n;
     }
@@ -391,8 +474,9 @@ cudaError_t launch_accept_parts(const float* logits, const int32_t* draft, int B
   const int parts = accept_parts(Bt, gamma, vocab, num_sms);
   const int vec4 = (vocab % 4 == 0) && ((reinterpret_cast<uintptr_t>(logits) & 15u) == 0);
   auto* keys = static_cast<unsigned long long*>(workspace);
-  cudaError_t e = launch_overlapped(accept_part_kernel, dim3(static_cast<unsigned>(Bt) * parts), dim3(kAcceptThreads),
-                                    0, stream, 1u, logits, gamma, vocab, vec4, parts, keys);
+  cudaError_t e = launch_overlapped(vec4 ? accept_part_kernel<true> : accept_part_kernel<false>,
+                                    dim3(static_cast<unsigned>(Bt) * parts), dim3(kAcceptThreads), 0, stream, 1u,
+                                    logits, gamma, vocab, parts, keys);
   if (e != cudaSuccess) return e;
   return launch_overlapped(accept_merge_kernel, dim3(static_cast<unsigned>(Bt)), dim3(kMergeThreads), 0, stream, 1u,
                            static_cast<const unsigned long long*>(keys), parts, draft, gamma, vocab, accepted_len,
@@ -412,9 +496,9 @@ cudaError_t launch_accept(const float* logits, const int32_t* draft, int Bt, int
     if (e != cudaSuccess) return e;
     if (cap->resident[kMaxCluster] >= Bt) {
       if (fault.extra) return cudaErrorNotSupported;
-      return launch_overlapped(accept_kernel<16>, dim3(static_cast<unsigned>(Bt) * kMaxCluster),
+      return launch_overlapped(vec4 ? accept_kernel<16, true> : accept_kernel<16, false>, dim3(static_cast<unsigned>(Bt) * kMaxCluster),
                                dim3(kAcceptThreads), 0, stream, static_cast<unsigned>(kMaxCluster), logits, draft,
-                               gamma, vocab, vec4, accepted_len, out_tokens, row_argmax, err_word, 0u, wait_ns);
+                               gamma, vocab, accepted_len, out_tokens, row_argmax, err_word, 0u, wait_ns);
     }
   }
   cudaError_t e = cluster_capacity<8>(&cap);
@@ -429,8 +513,8 @@ cudaError_t launch_accept(const float* logits, const int32_t* draft, int Bt, int
     }
   }
   if (fault.extra && CL > 1) return cudaErrorNotSupported;
-  return launch_overlapped(accept_kernel<8>, dim3(static_cast<unsigned>(Bt) * CL), dim3(kAcceptThreads), 0, stream,
-                           static_cast<unsigned>(CL), logits, draft, gamma, vocab, vec4, accepted_len, out_tokens,
+  return launch_overlapped(vec4 ? accept_kernel<8, true> : accept_kernel<8, false>, dim3(static_cast<unsigned>(Bt) * CL), dim3(kAcceptThreads), 0, stream,
+                           static_cast<unsigned>(CL), logits, draft, gamma, vocab, accepted_len, out_tokens,
                            row_argmax, err_word, fault.extra, wait_ns);
 }
 
