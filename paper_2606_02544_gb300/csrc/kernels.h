@@ -67,7 +67,7 @@ struct AttnF32Args {
   RopeTable rope;
   float* out;
   int32_t* err_word;
-  int num_pages, max_pages, page_size, Bt, gamma, Hq, Hkv, d;
+  int num_pages, max_pages, page_size, Bt, gamma, Hq, Hkv, d, num_sms;
   float scale;
 };
 cudaError_t launch_attention_f32(const AttnF32Args& a, cudaStream_t stream);

@@ -22,6 +22,8 @@ __global__ void __launch_bounds__(64) build_mask_kernel(const int32_t* __restric
   pdl_wait();
   pdl_launch_next();
   if (i == 0) map_ok = 1;
+  // (loaded beside the step map: one round trip to memory, not two in turn)
+  const int n = prefix_len[b];
   if (i < gamma) mu[i] = step_map ? step_map[static_cast<size_t>(b) * gamma + i] : i + 1;
   __syncthreads();
   // the drafted labels must be distinct values in 1..gamma; the other
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(64) build_mask_kernel(const int32_t* __restric
     tau[o] = t;
     section[o] = sec;
     // RoPE copy: D~_k reuses the position of D_k, which is n_b + k
-    rope_pos[o] = prefix_len[b] + k;
+    rope_pos[o] = n + k;
   }
   __syncthreads();
   if (mask_bits && i < S) {
