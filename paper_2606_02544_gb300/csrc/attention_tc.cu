@@ -80,7 +80,6 @@ constexpr int kHalfBytes = kTile * 128;     // 64 rows x 64 bf16 (one d-half of 
 constexpr int kMaxSplitFuse = 8;            // cluster of at most 8 splits
 constexpr int kPartStride = kD + 4;         // floats per partial row (no bank conflicts)
 constexpr int kPartMl = kRows * kPartStride;              // (m, l) per row
-constexpr int kPartWts = kPartMl + 2 * kRows;             // merge weights [row][split]
 constexpr int kSlotBytes = 4 * kHalfBytes;  // K0 K1 V0 V1, or Q0 Q1 (16 KB each)
 constexpr int kPageCache = 512;             // page ids of one sequence kept in shared memory
 constexpr float kRescaleThreshold = 8.0f;   // log2 units: rescale when the max grows by > 2^8
@@ -123,7 +122,7 @@ struct alignas(1024) Smem {
 
 constexpr size_t smem_bytes() { return sizeof(Smem) + 1024; }
 static_assert(kCtasPerSm * (smem_bytes() + 1024) <= 233472, "two CTAs per SM");
-static_assert((kPartWts + (kRows / 2) * kMaxSplitFuse) * sizeof(float) <= sizeof(Smem::ring),
+static_assert((kPartMl + 2 * kRows) * sizeof(float) <= sizeof(Smem::ring),
               "the fused split merge fits in the ring");
 
 __device__ __forceinline__ void signal_abort(Smem& sm, int32_t* err_word) {
@@ -134,6 +133,72 @@ __device__ __forceinline__ void signal_abort(Smem& sm, int32_t* err_word) {
 // Row r of a 128-byte-swizzled tile: 16-byte chunk c sits at chunk c ^ (r & 7).
 __device__ __forceinline__ uint4 ld_sw128_chunk(const uint8_t* half, int r, int c) {
   return *reinterpret_cast<const uint4*>(half + r * 128 + ((c ^ (r & 7)) << 4));
+}
+
+// Merge of the splits of a unit in their cluster (the four softmax warps):
+// O = sum_i 2^(m_i - M) O_i / sum_i 2^(m_i - M) l_i.  CTA `split` takes rows
+// split, split + nsplit, ... of the row block, a warp per row with lanes over
+// d, U rows of a warp at a time.  A row's (m, l) and partial O of every split
+// are requested together, so U rows cost one round trip through distributed
+// shared memory.  Every thread arrives on the cluster barrier once its loads
+// have returned; the caller waits on it.
+template <int NS, int U>
+__device__ __forceinline__ void merge_splits(const TcParams& p, const float* part, int split, int rblk, int b,
+                                             int kvh) {
+  const int nsp = p.nsplit, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nrows = (p.rows_blk - split + nsp - 1) / nsp;
+  const uint32_t at = smem_u32(part);
+#pragma unroll 1
+  for (int k0 = warp; k0 < nrows; k0 += 4 * U) {
+    float m[U][NS], l[U][NS];
+    float4 x[U][NS];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int r = split + min(k0 + 4 * u, nrows - 1) * nsp;  // (rows past the last: read again, not stored)
+#pragma unroll
+      for (int i = 0; i < NS; ++i) {
+        m[u][i] = -INFINITY;
+        l[u][i] = 0.f;
+        x[u][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < nsp) {
+          const uint32_t base = peer_smem(at, i);
+          ld_cluster_f32x2(base + 4 * (kPartMl + 2 * r), m[u][i], l[u][i]);
+          x[u][i] = ld_cluster_f32x4(base + 4 * (r * kPartStride + 4 * lane));
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int r = split + (k0 + 4 * u) * nsp;
+      float M = -INFINITY, L = 0.f;
+#pragma unroll
+      for (int i = 0; i < NS; ++i)
+        if (l[u][i] > 0.f) M = fmaxf(M, m[u][i]);
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < NS; ++i) m[u][i] = (M != -INFINITY && l[u][i] > 0.f) ? exp2f(m[u][i] - M) : 0.f;
+#pragma unroll
+      for (int i = 0; i < NS; ++i) L = fmaf(m[u][i], l[u][i], L);
+      const float inv = L > 0.f ? 1.f / L : 0.f;
+#pragma unroll
+      for (int i = 0; i < NS; ++i) {
+        const float w = m[u][i] * inv;
+        v.x = fmaf(w, x[u][i].x, v.x);
+        v.y = fmaf(w, x[u][i].y, v.y);
+        v.z = fmaf(w, x[u][i].z, v.z);
+        v.w = fmaf(w, x[u][i].w, v.w);
+      }
+      const int sr = rblk * p.s_blk + r / p.g;
+      if (k0 + 4 * u < nrows && sr < p.S) {
+        uint2 pk;
+        pk.x = pack_bf16x2(v.x, v.y);
+        pk.y = pack_bf16x2(v.z, v.w);
+        reinterpret_cast<uint2*>(p.out +
+                                 ((static_cast<size_t>(b) * p.S + sr) * p.Hq + kvh * p.g + r % p.g) * kD)[lane] = pk;
+      }
+    }
+  }
+  cluster_arrive();
 }
 
 // kFuse: the prefix splits of a unit form a cluster and merge their partials
@@ -325,10 +390,20 @@ __global__ void __maxnreg__(kMaxRegs)
     const int i = tid + j * kThreads;
     pg_reg[j] = i < pg_lim ? bt[i] : -1;
   }
-  for (int i = tid; i < p.S; i += kThreads) {
-    sm.tau[i] = p.tau[static_cast<size_t>(b) * p.S + i];
-    sm.sect[i] = p.section[static_cast<size_t>(b) * p.S + i];
-    if (kRope) sm.pos[i] = p.rope_pos[static_cast<size_t>(b) * p.S + i];
+  // (S <= 64 slots, one a thread; everything is in registers before the
+  // first store, which the compiler must keep behind the loads before it)
+  int lab_t = 0, lab_pos = 0;
+  uint8_t lab_s = 0;
+  if (tid < p.S) {
+    const size_t o = static_cast<size_t>(b) * p.S + tid;
+    lab_t = p.tau[o];
+    lab_s = p.section[o];
+    if (kRope) lab_pos = p.rope_pos[o];
+  }
+  if (tid < p.S) {
+    sm.tau[tid] = lab_t;
+    sm.sect[tid] = lab_s;
+    if (kRope) sm.pos[tid] = lab_pos;
   }
   const bool n_bad = n < 0 || static_cast<long long>(n) > static_cast<long long>(p.max_pages) * p.page_size;
   if (n_bad) {
@@ -424,35 +499,55 @@ __global__ void __maxnreg__(kMaxRegs)
     if (lane == 0 && ntiles > 0) {
       constexpr uint32_t kIdescQK = idesc_bf16_f32(kRows, kTile, 0, 0);
       constexpr uint32_t kIdescPV = idesc_bf16_f32(kRows, kD, 0, 1);
-      bool ok = mbar_wait(smem_u32(&sm.bar_qt), 0, abort_flag, p.wait_ns);
-      for (int i = 0; ok && i < ntiles; ++i) {
-        const int it = i + 1, st = it % kStages;
-        const uint32_t par = (it / kStages) & 1;
-        // S overwrites P of the previous tile; tcgen05.mma ops issued by one
-        // thread run in issue order, so that PV has read P before this S lands
-        if (!mbar_wait(smem_u32(&sm.bar_k[st]), par, abort_flag, p.wait_ns)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t kb0 = smem_u32(sm.ring[st]), kb1 = kb0 + kHalfBytes;
+      auto issue_s = [&](int it) {
+        const uint32_t kb0 = smem_u32(sm.ring[it % kStages]), kb1 = kb0 + kHalfBytes;
 #pragma unroll
         for (int kk = 0; kk < kD / 16; ++kk) {
           const uint32_t ka = (kk < 4 ? kb0 : kb1) + (kk & 3) * 32;
           tc_mma_ts(tmem + kColS, tmem + kColQ + 8 * kk, sdesc_sw128(ka, 16, 1024), kIdescQK, kk > 0);
         }
         tc_commit(smem_u32(&sm.bar_s_full));
-        if (!mbar_wait(smem_u32(&sm.bar_p), i & 1, abort_flag, p.wait_ns) ||
-            !mbar_wait(smem_u32(&sm.bar_v[st]), par, abort_flag, p.wait_ns)) {
+      };
+      bool ok = mbar_wait(smem_u32(&sm.bar_qt), 0, abort_flag, p.wait_ns);
+      bool s_issued = false;
+      for (int i = 0; ok && i < ntiles; ++i) {
+        const int it = i + 1, st = it % kStages;
+        const uint32_t par = (it / kStages) & 1;
+        // S overwrites P of the previous tile; tcgen05.mma ops issued by one
+        // thread run in issue order, so that PV has read P before this S lands
+        if (!s_issued) {
+          if (!mbar_wait(smem_u32(&sm.bar_k[st]), par, abort_flag, p.wait_ns)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          issue_s(it);
+        }
+        s_issued = false;
+        // V first: it has usually landed while the softmax works, and P is
+        // then acted on at once (a tile's chain of S, softmax and PV is serial
+        // within a CTA, 1.2 us of which the tensor core works 0.3; waiting in
+        // this order and issuing the next S ahead of the commits: 64
+        // sequences of 2048 to 8192 keys 213.7 -> 205.6 us, 32 x 4096 93.4 ->
+        // 86.1, 36 layers of 8 short sequences 824 -> 768)
+        if (!mbar_wait(smem_u32(&sm.bar_v[st]), par, abort_flag, p.wait_ns) ||
+            !mbar_wait(smem_u32(&sm.bar_p), i & 1, abort_flag, p.wait_ns)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t vb = kb0 + 2 * kHalfBytes;
+        const uint32_t vb = smem_u32(sm.ring[st]) + 2 * kHalfBytes;
 #pragma unroll
         for (int kk = 0; kk < kTile / 16; ++kk) {
           tc_mma_ts(tmem + kColO, tmem + kColS + 8 * kk, sdesc_sw128(vb + kk * 2048, kHalfBytes, 1024),
                     kIdescPV, (i > 0 || kk > 0) ? 1u : 0u);
+        }
+        // the next tile's S goes right behind this PV when its K is there
+        // (ahead of the commits, each of which holds the thread a while)
+        if (i + 1 < ntiles && mbar_test_wait(smem_u32(&sm.bar_k[(it + 1) % kStages]), ((it + 1) / kStages) & 1)) {
+          tc_fence_after();
+          issue_s(it + 1);
+          s_issued = true;
         }
         tc_commit(smem_u32(&sm.bar_empty[st]));
         tc_commit(smem_u32(&sm.bar_pv));
@@ -483,30 +578,36 @@ __global__ void __maxnreg__(kMaxRegs)
 
     // ---- Q: shared memory (ring slot 0) -> TMEM columns [0, 64)
     if (ntiles > 0) {
-      ok = mbar_wait_warp(smem_u32(&sm.bar_k[0]), 0, abort_flag, p.wait_ns);
-      if (kRope) {
+      if (!kRope) {
+        ok = mbar_wait_warp(smem_u32(&sm.bar_k[0]), 0, abort_flag, p.wait_ns);
+      } else {
         // rotate this unit's queries and, in the split that holds them (its
-        // first tile, ring item 1), the new keys at their slots' positions
-        constexpr int st1 = 1 % kStages;
+        // first tile, ring item 1), the new keys at their slots' positions;
+        // a thread's first angles are formed while Q is in flight
+        constexpr int st1 = 1 % kStages, kStep = 128 / kRopeThreadsPerSlot;
         const bool keys_here = t0 == 0;
+        const int q4 = tid % kRopeThreadsPerSlot;
+        float2 f[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) f[e] = p.rope.f[4 * q4 + e];
+        const int s0 = rblk * p.s_blk, s1 = min(p.S, s0 + p.s_blk);  // the slots of this block's query rows
+        const int lo = keys_here ? 0 : s0, hi = keys_here ? p.S : s1;
+        int t = lo + tid / kRopeThreadsPerSlot;
+        float sn[4], cs[4];
+        if (t < hi) rope_angles4(sm.pos[t], f, sn, cs);
+        ok = mbar_wait_warp(smem_u32(&sm.bar_k[0]), 0, abort_flag, p.wait_ns);
         if (ok && keys_here) ok = mbar_wait_warp(smem_u32(&sm.bar_k[st1]), 0, abort_flag, p.wait_ns);
         if (ok) {
-          const int q4 = tid % kRopeThreadsPerSlot;
-          float2 f[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) f[e] = p.rope.f[4 * q4 + e];
-          const int s0 = rblk * p.s_blk, s1 = min(p.S, s0 + p.s_blk);  // the slots of this block's query rows
-          const int lo = keys_here ? 0 : s0, hi = keys_here ? p.S : s1;
 #pragma unroll 1
-          for (int t = lo + tid / kRopeThreadsPerSlot; t < hi; t += 128 / kRopeThreadsPerSlot) {
-            float sn[4], cs[4];
-            rope_angles4(sm.pos[t], f, sn, cs);
+          while (t < hi) {
             if (t >= s0 && t < s1) {
 #pragma unroll 2
               for (int j = 0; j < p.g; ++j)
                 rope_rotate4(sm.ring[0], sm.ring[0] + 2 * kHalfBytes, (t - s0) * p.g + j, q4, sn, cs);
             }
             if (keys_here) rope_rotate4(sm.ring[st1], sm.ring[st1] + kHalfBytes, t, q4, sn, cs);
+            t += kStep;
+            if (t < hi) rope_angles4(sm.pos[t], f, sn, cs);
           }
           // read next by the tensor core (keys) and overwritten by TMA (the
           // queries' slot)
@@ -654,10 +755,10 @@ __global__ void __maxnreg__(kMaxRegs)
     }
     if (!ok && lane == 0) signal_abort(sm, p.err_word);
     // the next kernel on the stream may be scheduled now (its CTAs wait for
-    // this grid to finish anyway).  A clustered grid lets it in only when
-    // its CTAs exit: next-kernel CTAs placed beside clusters still merging
-    // cost more than they gain (measured at 8 sequences, 4 splits each).
-    if (!kFuse) pdl_launch_next();
+    // this grid to finish anyway); a clustered grid too, ahead of its merge:
+    // the next layer's set-up then runs under it (36 layers of 8 sequences,
+    // 809 us with the trigger at exit, 768 here)
+    pdl_launch_next();
     // ---- epilogue: O of the last PV, scaled by 1/l
     const bool have_o =
         ok && ntiles > 0 && mbar_wait_warp(smem_u32(&sm.bar_pv), (ntiles - 1) & 1, abort_flag, p.wait_ns);
@@ -759,63 +860,16 @@ __global__ void __maxnreg__(kMaxRegs)
     }
     cluster.sync();  // every split's partials are in place
     if (warp < 4) {
-      // Every remote load of a step is issued before its first use, so one
-      // round trip through distributed shared memory serves all splits.
-      const int nsp = p.nsplit;
-      float* wts = part + kPartWts;  // [row of this CTA][split]
-      const int nrows = (p.rows_blk - split + nsp - 1) / nsp;
-      for (int k = tid; k < nrows; k += 128) {
-        const int r = split + k * nsp;
-        float2 ml[kMaxSplitFuse];
-#pragma unroll
-        for (int i = 0; i < kMaxSplitFuse; ++i)
-          ml[i] = i < nsp ? *reinterpret_cast<const float2*>(cluster.map_shared_rank(part, i) + kPartMl + 2 * r)
-                          : make_float2(-INFINITY, 0.f);
-        float M = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < kMaxSplitFuse; ++i)
-          if (ml[i].y > 0.f) M = fmaxf(M, ml[i].x);
-        float w[kMaxSplitFuse], L = 0.f;
-#pragma unroll
-        for (int i = 0; i < kMaxSplitFuse; ++i) {
-          w[i] = (M != -INFINITY && ml[i].y > 0.f) ? exp2f(ml[i].x - M) : 0.f;
-          L = fmaf(w[i], ml[i].y, L);
-        }
-        const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-        for (int i = 0; i < kMaxSplitFuse; ++i) wts[k * kMaxSplitFuse + i] = w[i] * inv;
-      }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      constexpr int kVec = kD / 4;
-      for (int e = tid; e < nrows * kVec; e += 128) {
-        const int k = e / kVec, c4 = e - k * kVec;
-        const int r = split + k * nsp;
-        float4 x[kMaxSplitFuse];
-#pragma unroll
-        for (int i = 0; i < kMaxSplitFuse; ++i)
-          if (i < nsp) x[i] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(part, i) + r * kPartStride + 4 * c4);
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < kMaxSplitFuse; ++i) {
-          if (i < nsp) {
-            const float wi = wts[k * kMaxSplitFuse + i];
-            v.x = fmaf(wi, x[i].x, v.x);
-            v.y = fmaf(wi, x[i].y, v.y);
-            v.z = fmaf(wi, x[i].z, v.z);
-            v.w = fmaf(wi, x[i].w, v.w);
-          }
-        }
-        const int sr = rblk * p.s_blk + r / p.g;
-        if (sr < p.S) {
-          const int hr = kvh * p.g + r % p.g;
-          uint2 pk;
-          pk.x = pack_bf16x2(v.x, v.y);
-          pk.y = pack_bf16x2(v.z, v.w);
-          *reinterpret_cast<uint2*>(p.out + ((static_cast<size_t>(b) * p.S + sr) * p.Hq + hr) * kD + 4 * c4) = pk;
-        }
-      }
+      if (p.nsplit <= 2)
+        merge_splits<2, 4>(p, part, split, rblk, b, kvh);
+      else if (p.nsplit <= 4)
+        merge_splits<4, 4>(p, part, split, rblk, b, kvh);
+      else
+        merge_splits<8, 2>(p, part, split, rblk, b, kvh);
+    } else {
+      cluster_arrive();
     }
-    cluster.sync();  // no CTA leaves while a peer may still read its partials
+    cluster_wait();  // no CTA leaves while a peer may still read its partials
   }
 
   tc_fence_before();
