@@ -1,4 +1,5 @@
 // attention_tc.cu -- bf16 verification attention on the sm_103a tensor cores
+// (row blocks of more than 64 query rows; up to 64 go to attention_tc64.cu)
 // (Sec. 3.2 "Target Model Verification", Sec. 3.3 KV cache; the extra cost
 // of the paired layout is linear in the prefix, Eqs. (4)-(5)).
 //
@@ -41,9 +42,7 @@
 #include <algorithm>
 #include <mutex>
 
-#include "common.cuh"
-#include "kernels.h"
-#include "ptx.cuh"
+#include "attention_tc.cuh"
 #include "rope_tile.cuh"
 
 // Scratch of simsd_verify_attention_noalloc: the split partials live in this
@@ -58,9 +57,6 @@ namespace cg = cooperative_groups;
 namespace simsd {
 namespace {
 
-constexpr int kTile = 64;            // keys per tile
-constexpr int kD = 128;              // head dimension
-constexpr int kRows = 128;           // MMA M (query rows per CTA)
 constexpr int kStages = 3;           // ring slots of one CTA
 constexpr int kThreads = 192;
 constexpr int kCtasPerSm = 2;        // shared-memory budget of one CTA
@@ -75,36 +71,7 @@ constexpr int kWarpProducer = 4;
 constexpr int kWarpMma = 5;
 constexpr uint32_t kTmemCols = 256;
 constexpr uint32_t kColQ = 0, kColS = 64, kColO = 128;
-constexpr int kHalfBytes = kTile * 128;     // 64 rows x 64 bf16 (one d-half of K or V)
-// Split merge in place (fused): per-row partials in the ring, padded rows
-constexpr int kMaxSplitFuse = 8;            // cluster of at most 8 splits
-constexpr int kPartStride = kD + 4;         // floats per partial row (no bank conflicts)
-constexpr int kPartMl = kRows * kPartStride;              // (m, l) per row
 constexpr int kSlotBytes = 4 * kHalfBytes;  // K0 K1 V0 V1, or Q0 Q1 (16 KB each)
-constexpr int kPageCache = 512;             // page ids of one sequence kept in shared memory
-constexpr float kRescaleThreshold = 8.0f;   // log2 units: rescale when the max grows by > 2^8
-
-struct TcParams {
-  const int32_t* block_table;
-  const int32_t* prefix_len;
-  const int32_t* tau;
-  const uint8_t* section;
-  const int32_t* rope_pos;  // [Bt][2*gamma] or null (inputs rotated already)
-  __nv_bfloat16* out;
-  float* ws;  // partials: O [units*nsplit][rows_blk][128] then (m, l) [units*nsplit][rows_blk][2]
-  int32_t* err_word;
-  int max_pages, page_size, num_pages;
-  int Bt, gamma, S, Hq, Hkv, g, rb, rows_blk, s_blk, nsplit;
-  int sort;  // order sequences longest prefix first (grids of more than one wave)
-  int slots;  // CTAs resident at once: blocks past this start in a later wave
-  int fuse;   // the prefix splits of a unit form a cluster and merge in shared memory
-  float scale_log2;
-  // bounded waits: time limit and extra arrivals expected on bar_p (0 in
-  // normal use; a test arms one launch so that a wait runs out)
-  unsigned long long wait_ns;
-  uint32_t extra_p;
-  RopeTable rope;
-};
 
 struct alignas(1024) Smem {
   uint8_t ring[kStages][kSlotBytes];
@@ -122,7 +89,7 @@ struct alignas(1024) Smem {
 
 constexpr size_t smem_bytes() { return sizeof(Smem) + 1024; }
 static_assert(kCtasPerSm * (smem_bytes() + 1024) <= 233472, "two CTAs per SM");
-static_assert((kPartMl + 2 * kRows) * sizeof(float) <= sizeof(Smem::ring),
+static_assert((kPartWts + kRows / 2 * kWtsStride) * sizeof(float) <= sizeof(Smem::ring),
               "the fused split merge fits in the ring");
 
 __device__ __forceinline__ void signal_abort(Smem& sm, int32_t* err_word) {
@@ -133,72 +100,6 @@ __device__ __forceinline__ void signal_abort(Smem& sm, int32_t* err_word) {
 // Row r of a 128-byte-swizzled tile: 16-byte chunk c sits at chunk c ^ (r & 7).
 __device__ __forceinline__ uint4 ld_sw128_chunk(const uint8_t* half, int r, int c) {
   return *reinterpret_cast<const uint4*>(half + r * 128 + ((c ^ (r & 7)) << 4));
-}
-
-// Merge of the splits of a unit in their cluster (the four softmax warps):
-// O = sum_i 2^(m_i - M) O_i / sum_i 2^(m_i - M) l_i.  CTA `split` takes rows
-// split, split + nsplit, ... of the row block, a warp per row with lanes over
-// d, U rows of a warp at a time.  A row's (m, l) and partial O of every split
-// are requested together, so U rows cost one round trip through distributed
-// shared memory.  Every thread arrives on the cluster barrier once its loads
-// have returned; the caller waits on it.
-template <int NS, int U>
-__device__ __forceinline__ void merge_splits(const TcParams& p, const float* part, int split, int rblk, int b,
-                                             int kvh) {
-  const int nsp = p.nsplit, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nrows = (p.rows_blk - split + nsp - 1) / nsp;
-  const uint32_t at = smem_u32(part);
-#pragma unroll 1
-  for (int k0 = warp; k0 < nrows; k0 += 4 * U) {
-    float m[U][NS], l[U][NS];
-    float4 x[U][NS];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int r = split + min(k0 + 4 * u, nrows - 1) * nsp;  // (rows past the last: read again, not stored)
-#pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        m[u][i] = -INFINITY;
-        l[u][i] = 0.f;
-        x[u][i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < nsp) {
-          const uint32_t base = peer_smem(at, i);
-          ld_cluster_f32x2(base + 4 * (kPartMl + 2 * r), m[u][i], l[u][i]);
-          x[u][i] = ld_cluster_f32x4(base + 4 * (r * kPartStride + 4 * lane));
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int r = split + (k0 + 4 * u) * nsp;
-      float M = -INFINITY, L = 0.f;
-#pragma unroll
-      for (int i = 0; i < NS; ++i)
-        if (l[u][i] > 0.f) M = fmaxf(M, m[u][i]);
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int i = 0; i < NS; ++i) m[u][i] = (M != -INFINITY && l[u][i] > 0.f) ? exp2f(m[u][i] - M) : 0.f;
-#pragma unroll
-      for (int i = 0; i < NS; ++i) L = fmaf(m[u][i], l[u][i], L);
-      const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        const float w = m[u][i] * inv;
-        v.x = fmaf(w, x[u][i].x, v.x);
-        v.y = fmaf(w, x[u][i].y, v.y);
-        v.z = fmaf(w, x[u][i].z, v.z);
-        v.w = fmaf(w, x[u][i].w, v.w);
-      }
-      const int sr = rblk * p.s_blk + r / p.g;
-      if (k0 + 4 * u < nrows && sr < p.S) {
-        uint2 pk;
-        pk.x = pack_bf16x2(v.x, v.y);
-        pk.y = pack_bf16x2(v.z, v.w);
-        reinterpret_cast<uint2*>(p.out +
-                                 ((static_cast<size_t>(b) * p.S + sr) * p.Hq + kvh * p.g + r % p.g) * kD)[lane] = pk;
-      }
-    }
-  }
-  cluster_arrive();
 }
 
 // kFuse: the prefix splits of a unit form a cluster and merge their partials
@@ -860,12 +761,7 @@ __global__ void __maxnreg__(kMaxRegs)
     }
     cluster.sync();  // every split's partials are in place
     if (warp < 4) {
-      if (p.nsplit <= 2)
-        merge_splits<2, 4>(p, part, split, rblk, b, kvh);
-      else if (p.nsplit <= 4)
-        merge_splits<4, 4>(p, part, split, rblk, b, kvh);
-      else
-        merge_splits<8, 2>(p, part, split, rblk, b, kvh);
+      merge_unit(p, part, split, rblk, b, kvh);
     } else {
       cluster_arrive();
     }
@@ -1151,6 +1047,11 @@ cudaError_t launch_attention_tc(const AttnTcArgs& a, const AttnTcPlan& pl, Encod
     if (e != cudaSuccess) return e;
   }
   const long long grid = static_cast<long long>(a.Bt) * pl.nsplit * a.Hkv * pl.rb;
+  if (pl.rows_blk <= kTc64Rows) {
+    cudaError_t e = launch_attention_tc64(tq, tkn, tvn, tkc, tvc, p, stream);
+    if (e != cudaSuccess || pl.nsplit == 1 || pl.fuse) return e;
+    return launch_combine(p, static_cast<long long>(a.Bt) * a.Hkv * pl.rb * pl.rows_blk, pl.num_sms, stream);
+  }
   auto kern = a.rope_pos ? (pl.fuse ? attention_tc_kernel<true, true> : attention_tc_kernel<false, true>)
                          : (pl.fuse ? attention_tc_kernel<true, false> : attention_tc_kernel<false, false>);
   cudaError_t e = launch_overlapped(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreads), smem_bytes(), stream,
