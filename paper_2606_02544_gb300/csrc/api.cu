@@ -220,12 +220,19 @@ int verify_attention_impl(int dtype, const void* q, const void* k_new, const voi
 namespace simsd {
 
 RopeTable make_rope_table(double theta, int d) {
-  RopeTable t{};
+  // (64 calls of pow, about 3 us: a thread's layers ask for the same table)
+  thread_local RopeTable t{};
+  thread_local double t_theta = 0.0;
+  thread_local int t_d = 0;
+  if (theta == t_theta && d == t_d) return t;
+  t = RopeTable{};
   for (int i = 0; i < d / 2 && i < 64; ++i) {
     const double f = std::pow(theta, -2.0 * i / d) / 3.14159265358979323846;
     const float hi = static_cast<float>(f);
     t.f[i] = make_float2(hi, static_cast<float>(f - static_cast<double>(hi)));
   }
+  t_theta = theta;
+  t_d = d;
   return t;
 }
 

@@ -47,6 +47,8 @@ def load_library(path: str = LIB_PATH):
     """Loads libsimsd.so once; raises if it is missing (build it with
     ``paper_2606_02544_gb300.build.build()``)."""
     global _lib
+    if _lib is not None:  # (set once, under the lock)
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(path):
@@ -83,13 +85,23 @@ def load_library(path: str = LIB_PATH):
     return _lib
 
 
+# The raw handle of a device's current stream: what
+# torch.cuda.current_stream(device).cuda_stream returns, without the Stream
+# object in between (about 1 us of a call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    # (an int: ctypes converts it by the function's argtypes)
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _check(rc, where):
