@@ -780,10 +780,8 @@ __global__ void __maxnreg__(kMaxRegs)
 // O = sum_i 2^(m_i - M) O_i / sum_i 2^(m_i - M) l_i.  One warp per row; the
 // lanes take the splits' (m, l) in parallel, then sum the partial O rows with
 // lanes over the head dimension (independent loads, several in flight).
-// kBatch: splits whose partials a lane loads before adding any (see
-// launch_combine for the choice)
-template <int kBatch>
 __global__ void __launch_bounds__(128) combine_kernel(const __grid_constant__ TcParams p) {
+  constexpr int kBatch = 4;  // splits whose partials a lane loads before adding any
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const unsigned full = 0xffffffffu;
@@ -856,6 +854,83 @@ __global__ void __launch_bounds__(128) combine_kernel(const __grid_constant__ Tc
   // the next kernel is let in only as this grid's blocks finish: launched
   // at the start, its CTAs took SMs that thousands of these small blocks
   // still needed
+  pdl_launch_next();
+}
+
+// The same for many splits of few rows: a block per row, its four warps taking
+// the splits in turn (warp w: w, w + 4, ...; at most kRowPer each).  Every
+// partial of the row and every (m, l) is requested at once, each warp folds
+// its splits under its own maximum, and the four results are merged in shared
+// memory: one round trip to memory.  A warp per row walked the (m, l) twice
+// and the partials in batches of 16, four or five dependent round trips.
+constexpr int kRowPer = 16;
+__global__ void __launch_bounds__(128) combine_row_kernel(const __grid_constant__ TcParams p) {
+  __shared__ float4 acc_s[4][32];
+  __shared__ float m_s[4], l_s[4];
+  pdl_wait();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned full = 0xffffffffu;
+  const int row = static_cast<int>(blockIdx.x % p.rows_blk);
+  const unsigned u = blockIdx.x / p.rows_blk;
+  const int rblk = static_cast<int>(u % p.rb);
+  const int kvh = static_cast<int>((u / p.rb) % p.Hkv);
+  const int b = static_cast<int>(u / (static_cast<unsigned>(p.rb) * p.Hkv));
+  const int s = rblk * p.s_blk + row / p.g;
+  if (s >= p.S) return;  // (the same for the whole block)
+  const size_t units = static_cast<size_t>(p.Bt) * p.Hkv * p.rb, e0 = static_cast<size_t>(u) * p.nsplit;
+  const float2* wml = reinterpret_cast<const float2*>(p.ws + units * p.nsplit * p.rows_blk * kD);
+  const int cnt = (p.nsplit - warp + 3) / 4;  // this warp's splits
+  // lane j: (m, l) of split warp + 4 j
+  const float2 ml = lane < cnt ? wml[(e0 + warp + 4 * lane) * p.rows_blk + row] : make_float2(-INFINITY, 0.f);
+  float4 x[kRowPer];
+#pragma unroll
+  for (int j = 0; j < kRowPer; ++j)
+    x[j] = j < cnt ? reinterpret_cast<const float4*>(p.ws + ((e0 + warp + 4 * j) * p.rows_blk + row) * kD)[lane]
+                   : make_float4(0.f, 0.f, 0.f, 0.f);
+  float M = ml.y > 0.f ? ml.x : -INFINITY;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(full, M, o));
+  M = __shfl_sync(full, M, 0);
+  const float w = ml.y > 0.f ? exp2f(ml.x - M) : 0.f;
+  float L = w * ml.y;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) L += __shfl_xor_sync(full, L, o);
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int j = 0; j < kRowPer; ++j) {
+    const float wj = __shfl_sync(full, w, j);
+    acc.x = fmaf(wj, x[j].x, acc.x);
+    acc.y = fmaf(wj, x[j].y, acc.y);
+    acc.z = fmaf(wj, x[j].z, acc.z);
+    acc.w = fmaf(wj, x[j].w, acc.w);
+  }
+  acc_s[warp][lane] = acc;
+  if (lane == 0) {
+    m_s[warp] = M;
+    l_s[warp] = L;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    float Ma = m_s[0], La = 0.f;
+#pragma unroll
+    for (int k = 1; k < 4; ++k) Ma = fmaxf(Ma, m_s[k]);
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float f = l_s[k] > 0.f ? exp2f(m_s[k] - Ma) : 0.f;
+      const float4 v = acc_s[k][lane];
+      La = fmaf(f, l_s[k], La);
+      y.x = fmaf(f, v.x, y.x);
+      y.y = fmaf(f, v.y, y.y);
+      y.z = fmaf(f, v.z, y.z);
+      y.w = fmaf(f, v.w, y.w);
+    }
+    const float inv = La > 0.f ? 1.f / La : 0.f;
+    const int h = kvh * p.g + row % p.g;
+    reinterpret_cast<uint2*>(p.out + ((static_cast<size_t>(b) * p.S + s) * p.Hq + h) * kD)[lane] =
+        make_uint2(pack_bf16x2(y.x * inv, y.y * inv), pack_bf16x2(y.z * inv, y.w * inv));
+  }
+  // (the next kernel is let in as this grid's blocks finish, as above)
   pdl_launch_next();
 }
 
@@ -953,16 +1028,15 @@ bool plan_attention_tc(int Bt, int gamma, int Hq, int Hkv, int max_pages, int pa
   return true;
 }
 
-// The combine launch, a warp per row.  With many splits a row (a small
-// batch) a lane loads 16 splits' partials at once: 128 registers, four
-// blocks per SM, which pays while the grid fits in one wave of those.
-// Otherwise four at a time (about 56 registers): a large grid merging a
-// few splits a row needs its blocks resident more than wide loads.
-cudaError_t launch_combine(const TcParams& p, long long warps, int num_sms, cudaStream_t stream) {
-  const long long blocks = (warps + 3) / 4;
-  const bool wide = p.nsplit > 4 && blocks <= 4LL * num_sms;
-  return wide ? launch_overlapped(combine_kernel<16>, dim3(static_cast<unsigned>(blocks)), dim3(128), 0, stream, 1, p)
-              : launch_overlapped(combine_kernel<4>, dim3(static_cast<unsigned>(blocks)), dim3(128), 0, stream, 1, p);
+// The combine launch: a block per row for more than 4 splits of few rows (a
+// small batch), a warp per row otherwise (a large grid merging a few splits a
+// row needs its blocks resident more than loads in flight).  The whole call at
+// one sequence, 38 splits of each row, a warp a row -> a block a row: 32768
+// keys 35.4 -> 32.6 us, 8192 keys 18.4 -> 15.2.
+cudaError_t launch_combine(const TcParams& p, long long rows, int num_sms, cudaStream_t stream) {
+  if (p.nsplit > 4 && p.nsplit <= 4 * kRowPer && rows <= 16LL * num_sms)
+    return launch_overlapped(combine_row_kernel, dim3(static_cast<unsigned>(rows)), dim3(128), 0, stream, 1, p);
+  return launch_overlapped(combine_kernel, dim3(static_cast<unsigned>((rows + 3) / 4)), dim3(128), 0, stream, 1, p);
 }
 
 cudaError_t launch_attention_combine(const AttnTcArgs& a, const AttnTcPlan& pl, cudaStream_t stream) {
