@@ -230,16 +230,10 @@ __global__ void __maxnreg__(kF32Regs)
   float* ps = smem + L::p(W) + warp * kF32Keys * kF32Rows;  // this warp's P
   // rows of this warp that have an output to compute, and what they see of
   // the new slots (lane i < 8: row i)
-  unsigned long long vis = 0ull;
-  bool act = false;
-  if (lane < kF32Rows && row0 + lane < R && !seq_bad) {
-    const int s = (row0 + lane) / g;
-    const uint8_t si = lab_sect[s];
-    act = si != kSectPad;
-    if (act)
-      for (int t = 0; t < S; ++t)
-        if (temporal_visible(si, lab_tau[s], lab_sect[t], lab_tau[t])) vis |= 1ull << t;
-  }
+  const int own_row = row0 + min(lane, kF32Rows - 1), own_slot = own_row / g;
+  unsigned long long vis = slot_visibility(lab_tau, lab_sect, S, own_slot);
+  const bool act = lane < kF32Rows && own_row < R && !seq_bad && lab_sect[min(own_slot, S - 1)] != kSectPad;
+  if (!act) vis = 0ull;
   act_rows = __ballot_sync(full, act);
   bool ok = mbar_wait_warp(smem_u32(&bar_q), 0, abort_flag);
   if (row0 + kF32Rows > R) {

@@ -466,13 +466,8 @@ __global__ void __maxnreg__(kMaxRegs)
     const int hl = row % p.g;
     const bool row_exists = row < p.rows_blk && s < p.S;
     const bool active = row_exists && !seq_bad && sm.sect[s] != kSectPad;
-    unsigned long long vis = 0ull;
-    if (active) {
-      const uint8_t si = sm.sect[s];
-      const int ti = sm.tau[s];
-      for (int t = 0; t < p.S; ++t)
-        if (temporal_visible(si, ti, sm.sect[t], sm.tau[t])) vis |= 1ull << t;
-    }
+    unsigned long long vis = slot_visibility(sm.tau, sm.sect, p.S, s);
+    if (!active) vis = 0ull;
     const uint32_t lane_tmem = tmem + (static_cast<uint32_t>(warp * 32) << 16);
     float m_ref = -INFINITY, l_sum = 0.f;
     bool ok = true;
@@ -674,7 +669,7 @@ __global__ void __maxnreg__(kMaxRegs)
       fz_l = l_sum;
     } else if (p.nsplit == 1) {
       const float inv = any ? 1.0f / l_sum : 0.f;
-      __nv_bfloat16* orow = p.out + ((static_cast<size_t>(b) * p.S + s) * p.Hq + h) * kD;
+      const int at = row_exists ? (b * p.S + s) * p.Hq + h : -1;
 #pragma unroll 1
       for (int ch = 0; ch < kD / 32; ++ch) {
         uint32_t o[32];
@@ -682,25 +677,14 @@ __global__ void __maxnreg__(kMaxRegs)
           tmem_ld32(lane_tmem + kColO + 32 * ch, o);
           tmem_wait_ld();
         }
-        if (row_exists) {
-          uint4 pkd[4];
-          uint32_t* wv = reinterpret_cast<uint32_t*>(pkd);
-#pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            const float r0 = any ? __uint_as_float(o[2 * c]) * inv : 0.f;
-            const float r1 = any ? __uint_as_float(o[2 * c + 1]) * inv : 0.f;
-            wv[c] = pack_bf16x2(r0, r1);
-          }
-          uint4* dst = reinterpret_cast<uint4*>(orow + 32 * ch);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) dst[c] = pkd[c];
-        }
+        store_chunk_bf16(o, any, inv, p.out, at, ch);
       }
     } else {
       const size_t unit = ((static_cast<size_t>(b) * p.Hkv + kvh) * p.rb + rblk) * p.nsplit + split;
       const size_t nunits = static_cast<size_t>(p.Bt) * p.Hkv * p.rb * p.nsplit;
-      float* wo = p.ws + (unit * p.rows_blk + row) * kD;
+      float* wo = p.ws + unit * p.rows_blk * kD;
       float* wml = p.ws + nunits * p.rows_blk * kD + (unit * p.rows_blk + row) * 2;
+      const int at = row < p.rows_blk ? row : -1;
 #pragma unroll 1
       for (int ch = 0; ch < kD / 32; ++ch) {
         uint32_t o[32];
@@ -708,14 +692,7 @@ __global__ void __maxnreg__(kMaxRegs)
           tmem_ld32(lane_tmem + kColO + 32 * ch, o);
           tmem_wait_ld();
         }
-        if (row < p.rows_blk) {
-          float4* dst = reinterpret_cast<float4*>(wo + 32 * ch);
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            dst[c] = any ? make_float4(__uint_as_float(o[4 * c]), __uint_as_float(o[4 * c + 1]),
-                                       __uint_as_float(o[4 * c + 2]), __uint_as_float(o[4 * c + 3]))
-                         : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        store_chunk_f32(o, any, wo, at, ch);
       }
       if (row < p.rows_blk) {
         wml[0] = any ? m_ref : -INFINITY;

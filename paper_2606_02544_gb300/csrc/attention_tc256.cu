@@ -626,13 +626,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int s = x * p.s_blk + row / p.g;
       const bool row_exists = s < p.S;
       const bool active = row_exists && !seq_bad && sm.sect[par][s] != kSectPad;
-      unsigned long long vis = 0ull;
-      if (active) {
-        const uint8_t si = sm.sect[par][s];
-        const int ti = sm.tau[par][s];
-        for (int t = 0; t < p.S; ++t)
-          if (temporal_visible(si, ti, sm.sect[par][t], sm.tau[par][t])) vis |= 1ull << t;
-      }
+      unsigned long long vis = slot_visibility(sm.tau[par], sm.sect[par], p.S, s);
+      if (!active) vis = 0ull;
       float m_ref = -INFINITY, l_sum = 0.f;
       if (u.tiles > 0) {
         ++jq;
@@ -815,10 +810,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool any = have_o && active && l_sum > 0.f;
         const float inv = any ? 1.0f / l_sum : 0.f;
         const int h = u.kvh * p.g + hl;
-        __nv_bfloat16* orow = p.out + ((static_cast<size_t>(u.b) * p.S + (row_exists ? s : 0)) * p.Hq + h) * kD;
         // a split unit leaves its partial O (fp32) and (m, l) to the combine
         const bool part = u.part;
-        float* wo = part ? partial_o(p, u, x, row) : nullptr;
+        float* wo = part ? partial_o(p, u, x, 0) : nullptr;
+        const int at = !row_exists ? -1 : part ? row : (u.b * p.S + s) * p.Hq + h;
 #pragma unroll 1
         for (int ch = 0; ch < kD / 32; ++ch) {
           uint32_t o[32];
@@ -826,26 +821,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             tmem_ld32(o_tmem + 32 * ch, o);
             tmem_wait_ld();
           }
-          if (row_exists && part) {
-            float4* dst = reinterpret_cast<float4*>(wo + 32 * ch);
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-              dst[c] = any ? make_float4(__uint_as_float(o[4 * c]), __uint_as_float(o[4 * c + 1]),
-                                         __uint_as_float(o[4 * c + 2]), __uint_as_float(o[4 * c + 3]))
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
-          } else if (row_exists) {
-            uint4 pkd[4];
-            uint32_t* wv = reinterpret_cast<uint32_t*>(pkd);
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              const float r0 = any ? __uint_as_float(o[2 * c]) * inv : 0.f;
-              const float r1 = any ? __uint_as_float(o[2 * c + 1]) * inv : 0.f;
-              wv[c] = pack_bf16x2(r0, r1);
-            }
-            uint4* dst = reinterpret_cast<uint4*>(orow + 32 * ch);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) dst[c] = pkd[c];
-          }
+          if (part)
+            store_chunk_f32(o, any, wo, at, ch);
+          else
+            store_chunk_bf16(o, any, inv, p.out, at, ch);
         }
         if (row_exists && part) {
           float* wml = partial_ml(p, u, x, row);

@@ -28,6 +28,29 @@ __host__ __device__ __forceinline__ bool temporal_visible(uint8_t si, int ti, ui
   return (sj == kSectData) == (tj < ti + bias);
 }
 
+// The visibility word of a row of slot `s` (bit t: new slot t < S <= 64), for
+// the 32 rows of a warp at once.  The slots of a warp's rows are consecutive:
+// for each of them lane j judges columns j and j + 32, and two ballots make
+// the word.  All lanes call it; rows past the last slot get 0.  (A row at a
+// time, each thread walking the S labels, cost 3.4 us at S = 64.)
+__device__ __forceinline__ unsigned long long slot_visibility(const int32_t* tau, const uint8_t* sect, int S, int s) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, j0 = lane, j1 = lane + 32;
+  const uint8_t c0 = j0 < S ? sect[j0] : kSectPad, c1 = j1 < S ? sect[j1] : kSectPad;
+  const int t0 = j0 < S ? tau[j0] : 0, t1 = j1 < S ? tau[j1] : 0;
+  const int lo = __shfl_sync(full, s, 0), hi = min(S - 1, __shfl_sync(full, s, 31));
+  unsigned long long vis = 0ull;
+#pragma unroll 2
+  for (int k = lo; k <= hi; ++k) {
+    const uint8_t sk = sect[k];
+    const int tk = tau[k];
+    const unsigned w0 = __ballot_sync(full, temporal_visible(sk, tk, c0, t0));
+    const unsigned w1 = __ballot_sync(full, temporal_visible(sk, tk, c1, t1));
+    if (k == s) vis = static_cast<unsigned long long>(w1) << 32 | w0;
+  }
+  return vis;
+}
+
 // ---- programmatic dependent launch.  Every kernel of the library is
 // launched so that it may start (set-up only) while the previous kernel on
 // the stream finishes: it calls pdl_wait() before it reads or writes any

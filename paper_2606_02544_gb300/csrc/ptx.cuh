@@ -369,4 +369,71 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return d;
 }
 
+// Transposes N x N 16-byte pieces among each group of N lanes (4 or 8):
+// afterwards piece i of lane j of the group is what was piece j of lane i.
+template <int N>
+__device__ __forceinline__ void transpose_pieces(uint4 (&v)[N]) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int m = 1; m < N; m <<= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      if (i & m) continue;
+      // lanes with bit m clear keep piece i and swap piece i | m for the
+      // other's piece i
+      uint4 x = up ? v[i] : v[i | m];
+      x.x = __shfl_xor_sync(full, x.x, m);
+      x.y = __shfl_xor_sync(full, x.y, m);
+      x.z = __shfl_xor_sync(full, x.z, m);
+      x.w = __shfl_xor_sync(full, x.w, m);
+      if (up)
+        v[i] = x;
+      else
+        v[i | m] = x;
+    }
+  }
+}
+
+// 32 columns (chunk ch) of O, a row per lane, to rows of 128 columns at dst; at:
+// the row's index there, -1 for none (any false: the row is zero).  Four lanes
+// exchange 16-byte pieces first, so that a store covers 64-byte stretches of
+// eight rows; with every lane storing its own row a store
+// touched 32 lines (the 256-row kernel: 3.6 to 7 us a piece of 256 rows, 2.2 to 3
+// so).
+__device__ __forceinline__ void store_chunk_f32(const uint32_t (&o)[32], bool any, float* dst, int at, int ch) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    uint4 v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int k = 16 * q + 4 * c;
+      v[c] = any ? make_uint4(o[k], o[k + 1], o[k + 2], o[k + 3]) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    transpose_pieces<4>(v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int ai = __shfl_sync(0xffffffffu, at, (lane & ~3) + i);
+      if (ai >= 0) reinterpret_cast<uint4*>(dst)[static_cast<size_t>(ai) * 32 + 8 * ch + 4 * q + (lane & 3)] = v[i];
+    }
+  }
+}
+__device__ __forceinline__ void store_chunk_bf16(const uint32_t (&o)[32], bool any, float inv, void* dst, int at,
+                                                 int ch) {
+  const int lane = threadIdx.x & 31;
+  uint4 v[4];
+  uint32_t* wv = reinterpret_cast<uint32_t*>(v);
+#pragma unroll
+  for (int c = 0; c < 16; ++c)
+    wv[c] = pack_bf16x2(any ? __uint_as_float(o[2 * c]) * inv : 0.f, any ? __uint_as_float(o[2 * c + 1]) * inv : 0.f);
+  transpose_pieces<4>(v);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int ai = __shfl_sync(0xffffffffu, at, (lane & ~3) + i);
+    if (ai >= 0) reinterpret_cast<uint4*>(dst)[static_cast<size_t>(ai) * 16 + 4 * ch + (lane & 3)] = v[i];
+  }
+}
+
 }  // namespace simsd
