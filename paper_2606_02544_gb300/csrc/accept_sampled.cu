@@ -600,6 +600,9 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_part_kernel(const float*
   for (int i = tid; i < kSampWarps * kSampMaxRows; i += kSampThreads)
     part[i / kSampMaxRows][i % kSampMaxRows] = make_float2(kEmpty, 0.f);
   pdl_wait();
+  // (at once: the grid is one wave, so the waiting CTAs of samp_resid_kernel
+  // only take places that this one's CTAs have left)
+  pdl_launch_next();
   // the arrival count samp_resid_kernel uses for this sequence starts at 0
   if (c == 0 && tid == 0) arrivals[b] = 0u;
   __syncthreads();
@@ -611,7 +614,6 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_part_kernel(const float*
     for (int w = 0; w < kSampWarps; ++w) ms_merge(m, s, part[w][r].x, part[w][r].y);
     pre[(static_cast<size_t>(b) * parts + c) * rows + r] = make_float2(m, s);
   }
-  pdl_launch_next();
 }
 
 // Row a's weights at one unit of 4 columns (0 past the vocabulary): p_theta = 2^(z_t - m_t) / s_t and the residual
@@ -689,6 +691,7 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   const unsigned full = 0xffffffffu;
   pdl_wait();
   float zt = 0.f, zd = 0.f, ua = 0.f;
+  const float us = u_sample[b];
   bool bad = false;
   if (warp == 0 && lane < gamma) {
     const int x = draft[static_cast<size_t>(b) * gamma + lane];
@@ -786,12 +789,16 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   __threadfence();
   // ---- the last CTA of the sequence: which span holds the threshold
   if (warp == 0) {
-    // the other CTAs' sums, read past L1 (they were written by other SMs)
-    const volatile float* vs = reinterpret_cast<const volatile float*>(sums + static_cast<size_t>(b) * rparts);
-    float tr = 0.f, tt = 0.f;
-    for (int q = lane; q < rparts; q += 32) {
-      tr += vs[2 * q];
-      tt += vs[2 * q + 1];
+    // the other CTAs' sums, read past L1 (they were written by other SMs);
+    // the first two a lane stay in registers for the scan below
+    const float2* vs = sums + static_cast<size_t>(b) * rparts;
+    const float2 v0 = lane < rparts ? __ldcg(vs + lane) : make_float2(0.f, 0.f);
+    const float2 v1 = lane + 32 < rparts ? __ldcg(vs + lane + 32) : make_float2(0.f, 0.f);
+    float tr = v0.x + v1.x, tt = v0.y + v1.y;
+    for (int q = lane + 64; q < rparts; q += 32) {
+      const float2 v = __ldcg(vs + q);
+      tr += v.x;
+      tt += v.y;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -802,12 +809,15 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
     // the draw falls back to p_theta
     int mode = (resid && tr > kResidFloor) || (!resid && tr > 0.f) ? 0 : (tt > 0.f ? 1 : -1);
     const float total = mode == 0 ? tr : tt;
-    const float thr = u_sample[b] * total;
+    const float thr = us * total;
     int owner = -1, last_pos = -1;
     float base = 0.f, last_base = 0.f, run = 0.f;
     for (int q0 = 0; q0 < rparts && mode >= 0 && owner < 0; q0 += 32) {
       const int q = q0 + lane;
-      const float wq = q < rparts ? vs[2 * q + (mode == 0 ? 0 : 1)] : 0.f;
+      const float2 vq = q0 == 0    ? v0
+                        : q0 == 32 ? v1
+                                   : (q < rparts ? __ldcg(vs + q) : make_float2(0.f, 0.f));
+      const float wq = mode == 0 ? vq.x : vq.y;
       float incl = wq;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -852,8 +862,20 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   const int u0 = min(W, owner_sh * per), u1 = min(W, u0 + per);
   const int k = (u1 - u0 + kSampThreads - 1) / kSampThreads;
   const int t0 = min(u1, u0 + tid * k), t1 = min(u1, t0 + k);
+  // (the weights of the first two stay in registers for the walk: a span is at
+  // most 1024 units, two a thread, unless there are few parts)
+  const float4 kZero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 w0 = kZero, w1 = kZero;
+  if (t0 < t1) {
+    const int second = min(t0 + 1, t1 - 1);
+    const UnitW x0 = unit_weights<VEC>(rw, t0), x1 = unit_weights<VEC>(rw, second);
+    w0 = mode == 0 ? x0.r : x0.t;
+    if (t0 + 1 < t1) w1 = mode == 0 ? x1.r : x1.t;
+  }
   float mine = 0.f;
-  for (int u = t0; u < t1; ++u) {
+  mine += (w0.x + w0.y) + (w0.z + w0.w);
+  mine += (w1.x + w1.y) + (w1.z + w1.w);
+  for (int u = t0 + 2; u < t1; ++u) {
     const UnitW uw = unit_weights<VEC>(rw, u);
     const float4 w = mode == 0 ? uw.r : uw.t;
     mine += (w.x + w.y) + (w.z + w.w);
@@ -881,8 +903,11 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
     cum += w;
   };
   for (int u = t0; u < t1 && hit < 0; ++u) {
-    const UnitW uw = unit_weights<VEC>(rw, u);
-    const float4 w = mode == 0 ? uw.r : uw.t;
+    float4 w = u == t0 ? w0 : w1;
+    if (u > t0 + 1) {
+      const UnitW uw = unit_weights<VEC>(rw, u);
+      w = mode == 0 ? uw.r : uw.t;
+    }
     const int col = 4 * u;
     step(w.x, col);
     step(w.y, col + 1);
