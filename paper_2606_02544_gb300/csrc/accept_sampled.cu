@@ -601,7 +601,8 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_part_kernel(const float*
     part[i / kSampMaxRows][i % kSampMaxRows] = make_float2(kEmpty, 0.f);
   pdl_wait();
   // (at once: the grid is one wave, so the waiting CTAs of samp_resid_kernel
-  // only take places that this one's CTAs have left)
+  // only take places that this one's CTAs have left; with that kernel's loads
+  // issued ahead, 8 sequences of 9 rows of 151936 logits 24.9 -> 24.1 us)
   pdl_launch_next();
   // the arrival count samp_resid_kernel uses for this sequence starts at 0
   if (c == 0 && tid == 0) arrivals[b] = 0u;
@@ -616,8 +617,9 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_part_kernel(const float*
   }
 }
 
-// Row a's weights at one unit of 4 columns (0 past the vocabulary): p_theta = 2^(z_t - m_t) / s_t and the residual
-// max(0, p_theta - p_phi) (p_theta again when there is no draft row).
+// Row a's weights at one unit of 4 columns (0 past the vocabulary): p_theta =
+// 2^(z_t - m_t) / s_t and the residual max(0, p_theta - p_phi) (p_theta again
+// when there is no draft row).
 struct RowW {
   const float* trow;
   const float* drow;
