@@ -7,8 +7,8 @@
 //
 // One thread-block cluster per sequence.  Phase 1: the sequence's gamma+1
 // target rows and gamma draft rows are laid end to end, each row padded to a
-// multiple of 32 units (a unit is 16 bytes on a 16-byte boundary, whatever the
-// rows' own alignment), and the CTAs take contiguous spans of warp-aligned units, so the
+// multiple of 32 units (a unit is 4 floats, or 1 when rows are not 16-byte
+// aligned), and the CTAs take contiguous spans of warp-aligned units, so the
 // 32 lanes of a warp are always on the same row.  Each lane keeps the running maximum m of
 // z = x*log2(e)/T and s = sum 2^(z - m) of its row; when the warp moves to
 // the next row it merges its lanes by shuffles into a per-warp slot (no
@@ -96,41 +96,22 @@ __device__ __forceinline__ const float* row_ptr(const float* tgt, const float* d
                       : drf + (static_cast<size_t>(b) * gamma + (row - gamma - 1)) * vocab;
 }
 
-// Units of a row: 16-byte pieces.  VEC: every row starts on a 16-byte
-// boundary and holds a whole number of them.  Otherwise phase 1 takes the
-// aligned pieces that cover the row (one more than (vocab + 3) / 4 at most;
-// values outside the row count as -inf) and phase 2 four columns a unit.
+// the same through L1 (phase 2 re-reads a thread's lines)
 template <bool VEC>
-__host__ __device__ __forceinline__ constexpr int phase1_units(int vocab) {
-  return VEC ? vocab >> 2 : (vocab + 6) >> 2;
-}
-
-// Unit u of phase 2, columns 4 u .. 4 u + 3, through L1 (a thread's lines are
-// re-read)
-template <bool VEC>
-__device__ __forceinline__ float4 load_unit_cached(const float* rp, int u, int vocab) {
+__device__ __forceinline__ float4 load_unit_cached(const float* rp, int col) {
   if constexpr (VEC) {
-    return __ldg(reinterpret_cast<const float4*>(rp) + u);
+    return __ldg(reinterpret_cast<const float4*>(rp) + col);
   } else {
-    const int c = 4 * u;
-    return make_float4(__ldg(rp + c), c + 1 < vocab ? __ldg(rp + c + 1) : -INFINITY,
-                       c + 2 < vocab ? __ldg(rp + c + 2) : -INFINITY, c + 3 < vocab ? __ldg(rp + c + 3) : -INFINITY);
+    return make_float4(__ldg(rp + col), -INFINITY, -INFINITY, -INFINITY);
   }
 }
 
-// Unit `col` of phase 1.
 template <bool VEC>
-__device__ __forceinline__ float4 load_unit(const float* rp, int col, int vocab) {
+__device__ __forceinline__ float4 load_unit(const float* rp, int col) {
   if constexpr (VEC) {
     return ld_stream_f4(rp + 4 * col);
   } else {
-    // the first value's place in the row: rp - h is the 16-byte boundary
-    const int h = static_cast<int>((reinterpret_cast<uintptr_t>(rp) >> 2) & 3u), e = 4 * col - h;
-    if (e >= 0 && e + 3 < vocab) return ld_stream_f4(rp + e);
-    return make_float4(e >= 0 && e < vocab ? __ldg(rp + e) : -INFINITY,
-                       e + 1 >= 0 && e + 1 < vocab ? __ldg(rp + e + 1) : -INFINITY,
-                       e + 2 >= 0 && e + 2 < vocab ? __ldg(rp + e + 2) : -INFINITY,
-                       e + 3 >= 0 && e + 3 < vocab ? __ldg(rp + e + 3) : -INFINITY);
+    return make_float4(__ldg(rp + col), -INFINITY, -INFINITY, -INFINITY);
   }
 }
 
@@ -178,7 +159,7 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
   const int rows = 2 * gamma + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned full = 0xffffffffu;
-  const int W = phase1_units<VEC>(vocab);    // units per row
+  const int W = VEC ? (vocab >> 2) : vocab;  // units per row
   const int Wp = (W + 31) & ~31;             // padded: a warp never straddles two rows
   const int G = rows * (Wp >> 5);            // groups of 32 units
   const int per = (G + CL - 1) / CL;
@@ -222,7 +203,7 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
       // the common case: every unit valid, on one row, inside the row
 #pragma unroll
       for (int u = 0; u < H; ++u) {
-        v[u] = load_unit<VEC>(rp, col + u * kStep, vocab);
+        v[u] = load_unit<VEC>(rp, col + u * kStep);
         vr[u] = row;
       }
       advance(kStep * H);
@@ -232,7 +213,7 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
         vr[u] = -1;
         if (f + u * kStep < f1) {
           vr[u] = row;
-          v[u] = col < W ? load_unit<VEC>(rp, col, vocab) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+          v[u] = col < W ? load_unit<VEC>(rp, col) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         }
         advance(kStep);
       }
@@ -403,7 +384,7 @@ __global__ void __launch_bounds__(kSampThreads, UNROLL == 8 ? 2 : 1) accept_samp
   const float* drow = a < gamma ? drf + (static_cast<size_t>(b) * gamma + a) * vocab : trow;
   const float nmt = -row_m[a], it = 1.f / row_s[a];
   const float nmd = a < gamma ? -row_m[gamma + 1 + a] : 0.f, id = a < gamma ? 1.f / row_s[gamma + 1 + a] : 0.f;
-  const int W = (vocab + 3) >> 2;
+  const int W = VEC ? (vocab >> 2) : vocab;
   const int per_c = (W + CL - 1) / CL;
   const int c0 = min(W, c * per_c), c1 = min(W, c0 + per_c);
   const int per_w = (((c1 - c0 + kSampWarps - 1) / kSampWarps) + 31) & ~31;
@@ -411,7 +392,7 @@ __global__ void __launch_bounds__(kSampThreads, UNROLL == 8 ? 2 : 1) accept_samp
   const int nsteps = (w1 - w0 + 31) >> 5;
   const int M = max(1, (nsteps + kSampMacros - 1) / kSampMacros);
   const int nmac = (nsteps + M - 1) / M;
-  // the four weights of a unit
+  // the four weights of a unit (the scalar layout has one column per unit)
   auto weights = [&](const float4& xt, const float4& xd) -> float4 {
     float4 w = make_float4(ex2(fmaf(xt.x, zscale, nmt)) * it, ex2(fmaf(xt.y, zscale, nmt)) * it,
                            ex2(fmaf(xt.z, zscale, nmt)) * it, ex2(fmaf(xt.w, zscale, nmt)) * it);
@@ -430,8 +411,8 @@ __global__ void __launch_bounds__(kSampThreads, UNROLL == 8 ? 2 : 1) accept_samp
     for (int j = 0; j < 4; ++j) {
       const int u = w0 + 32 * (i0 + j) + lane;
       const bool ok = u < w1;
-      xt[j] = ok ? load_unit_cached<VEC>(trow, u, vocab) : kNone;
-      xd[j] = ok && resid ? load_unit_cached<VEC>(drow, u, vocab) : kNone;
+      xt[j] = ok ? load_unit_cached<VEC>(trow, u) : kNone;
+      xd[j] = ok && resid ? load_unit_cached<VEC>(drow, u) : kNone;
     }
   };
   // an empty residual (p_theta = p_phi to fp32 precision) cannot reject:
@@ -564,8 +545,8 @@ __global__ void __launch_bounds__(kSampThreads, UNROLL == 8 ? 2 : 1) accept_samp
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             if (w4[e] > 0.f) {
-              if (hit_col < 0 && cum + w4[e] > thr) hit_col = 4 * u + e;
-              pos_col = 4 * u + e;
+              if (hit_col < 0 && cum + w4[e] > thr) hit_col = VEC ? 4 * u + e : u;
+              pos_col = VEC ? 4 * u + e : u;
             }
             cum += w4[e];
           }
@@ -617,14 +598,13 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_part_kernel(const float*
   }
 }
 
-// Row a's weights at one unit of 4 columns (0 past the vocabulary): p_theta =
-// 2^(z_t - m_t) / s_t and the residual max(0, p_theta - p_phi) (p_theta again
-// when there is no draft row).
+// Row a's weights at one unit of 4 columns (1 in the scalar layout, the
+// other three 0): p_theta = 2^(z_t - m_t) / s_t and the residual
+// max(0, p_theta - p_phi) (p_theta again when there is no draft row).
 struct RowW {
   const float* trow;
   const float* drow;
   float zscale, nmt, it, nmd, id;
-  int vocab;
   bool resid;
 };
 struct UnitW {
@@ -632,12 +612,12 @@ struct UnitW {
 };
 template <bool VEC>
 __device__ __forceinline__ UnitW unit_weights(const RowW& w, int u) {
-  const float4 xt = load_unit_cached<VEC>(w.trow, u, w.vocab);
+  const float4 xt = load_unit_cached<VEC>(w.trow, u);
   UnitW o;
   o.t = make_float4(ex2(fmaf(xt.x, w.zscale, w.nmt)) * w.it, ex2(fmaf(xt.y, w.zscale, w.nmt)) * w.it,
                     ex2(fmaf(xt.z, w.zscale, w.nmt)) * w.it, ex2(fmaf(xt.w, w.zscale, w.nmt)) * w.it);
   if (w.resid) {
-    const float4 xd = load_unit_cached<VEC>(w.drow, u, w.vocab);
+    const float4 xd = load_unit_cached<VEC>(w.drow, u);
     o.r = make_float4(fmaxf(0.f, o.t.x - ex2(fmaf(xd.x, w.zscale, w.nmd)) * w.id),
                       fmaxf(0.f, o.t.y - ex2(fmaf(xd.y, w.zscale, w.nmd)) * w.id),
                       fmaxf(0.f, o.t.z - ex2(fmaf(xd.z, w.zscale, w.nmd)) * w.id),
@@ -712,7 +692,7 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   // of each of the warp's rows per round, all before any is merged
   {
     constexpr int kRowsPerWarp = (kSampMaxRows + kSampWarps - 1) / kSampWarps;
-    const int Wg = (phase1_units<VEC>(vocab) + 31) >> 5;  // groups per row
+    const int Wg = ((VEC ? (vocab >> 2) : vocab) + 31) >> 5;  // groups per row
     const int per = (rows * Wg + parts - 1) / parts;
     float m[kRowsPerWarp], sm[kRowsPerWarp];
     int q_lo[kRowsPerWarp], q_n[kRowsPerWarp];
@@ -766,9 +746,9 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   const float* drow = resid ? drf + (static_cast<size_t>(b) * gamma + a) * vocab : trow;
   const float nmt = -row_m[a], it = 1.f / row_s[a];
   const float nmd = resid ? -row_m[gamma + 1 + a] : 0.f, id = resid ? 1.f / row_s[gamma + 1 + a] : 0.f;
-  const int W = (vocab + 3) >> 2;
+  const int W = VEC ? (vocab >> 2) : vocab;
   const int per = (W + rparts - 1) / rparts;
-  const RowW rw{trow, drow, zscale, nmt, it, nmd, id, vocab, resid};
+  const RowW rw{trow, drow, zscale, nmt, it, nmd, id, resid};
   {
     const int u0 = min(W, c * per), u1 = min(W, u0 + per);
     float st = 0.f, sr = 0.f;
@@ -910,7 +890,7 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
       const UnitW uw = unit_weights<VEC>(rw, u);
       w = mode == 0 ? uw.r : uw.t;
     }
-    const int col = 4 * u;
+    const int col = VEC ? 4 * u : u;  // (the scalar layout's other three weights are 0)
     step(w.x, col);
     step(w.y, col + 1);
     step(w.z, col + 2);
