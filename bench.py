@@ -57,9 +57,9 @@ def _peaks():
 # the sources each stored traffic figure depends on: a kernel's own file and
 # the headers it includes
 TRAFFIC_SOURCES = {
-    "attention": ("attention_tc.cu", "ptx.cuh", "common.cuh"),
+    "attention": ("attention_tc.cu", "attention_tc64.cu", "attention_tc.cuh", "rope_tile.cuh", "ptx.cuh", "common.cuh"),
     "accept": ("accept.cu", "ptx.cuh", "common.cuh"),
-    "attention_tc256": ("attention_tc256.cu", "ptx.cuh", "common.cuh"),
+    "attention_tc256": ("attention_tc256.cu", "rope_tile.cuh", "ptx.cuh", "common.cuh"),
 }
 
 
