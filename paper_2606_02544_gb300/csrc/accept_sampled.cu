@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -107,11 +108,21 @@ __device__ __forceinline__ float4 load_unit_cached(const float* rp, int col) {
 }
 
 template <bool VEC>
-__device__ __forceinline__ float4 load_unit(const float* rp, int col) {
+using Unit = std::conditional_t<VEC, float4, float>;
+template <bool VEC>
+__device__ __forceinline__ Unit<VEC> load_unit(const float* rp, int col) {
   if constexpr (VEC) {
     return ld_stream_f4(rp + 4 * col);
   } else {
-    return make_float4(__ldg(rp + col), -INFINITY, -INFINITY, -INFINITY);
+    return __ldg(rp + col);
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ Unit<VEC> no_unit() {
+  if constexpr (VEC) {
+    return make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+  } else {
+    return -INFINITY;
   }
 }
 
@@ -152,7 +163,8 @@ __device__ __forceinline__ int accept_walk(int b, int gamma, int vocab, float zs
 // Phase 1 of one CTA: the running (m, s) of z = x log2(e) / T over span c
 // of CL equal spans of the sequence's rows (target rows 0..gamma, then
 // draft rows), merged per warp into part[warp][row].
-template <bool VEC, int UNROLL>
+// HS: scalar units loaded at a time.
+template <bool VEC, int UNROLL, int HS>
 __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const float* __restrict__ drf, int b,
                                             int gamma, int vocab, float zscale, int c, int CL,
                                             float2 (*part)[kSampMaxRows]) {
@@ -197,8 +209,11 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
   // Loads of H units.  f0, f1, Wp and the f and col of a warp's first lane
   // are multiples of 32, so every test here is the same for the 32 lanes
   // of a warp.  vr[u] is the unit's row, -1 past the span.
-  constexpr int H = UNROLL == 16 ? 8 : UNROLL;
-  auto fetch = [&](float4(&v)[H], int(&vr)[H]) {
+  // A scalar unit takes one register, so 16 are loaded at a time (8 before; the
+  // sums run in the same order): 32 sequences of 17 rows of 50001 logits 51.4 ->
+  // 45.7 us, 64 90.5 -> 79.0.
+  constexpr int H = VEC ? (UNROLL == 16 ? 8 : UNROLL) : HS;
+  auto fetch = [&](Unit<VEC>(&v)[H], int(&vr)[H]) {
     if (f - lane + kStep * (H - 1) < f1 && col - lane + kStep * (H - 1) + 31 < W) {
       // the common case: every unit valid, on one row, inside the row
 #pragma unroll
@@ -213,14 +228,14 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
         vr[u] = -1;
         if (f + u * kStep < f1) {
           vr[u] = row;
-          v[u] = col < W ? load_unit<VEC>(rp, col) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+          v[u] = col < W ? load_unit<VEC>(rp, col) : no_unit<VEC>();
         }
         advance(kStep);
       }
     }
     f += kStep * H;
   };
-  auto consume = [&](const float4(&v)[H], const int(&vr)[H]) {
+  auto consume = [&](const Unit<VEC>(&v)[H], const int(&vr)[H]) {
 #pragma unroll
     for (int u = 0; u < H; ++u) {
       if (vr[u] < 0) break;
@@ -230,20 +245,27 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
         m = kEmpty;
         s = 0.f;
       }
-      const float mz = fmaxf(fmaxf(v[u].x, v[u].y), fmaxf(v[u].z, v[u].w)) * zscale;
+      float mz;
+      if constexpr (VEC)
+        mz = fmaxf(fmaxf(v[u].x, v[u].y), fmaxf(v[u].z, v[u].w)) * zscale;
+      else
+        mz = fmaxf(v[u], -INFINITY) * zscale;  // (a NaN leaves the maximum alone)
       if (mz > m) {
         s *= ex2(m - mz);
         m = mz;
       }
       const float nm = -m;
-      s += ex2(fmaf(v[u].x, zscale, nm)) + ex2(fmaf(v[u].y, zscale, nm)) + ex2(fmaf(v[u].z, zscale, nm)) +
-           ex2(fmaf(v[u].w, zscale, nm));
+      if constexpr (VEC)
+        s += ex2(fmaf(v[u].x, zscale, nm)) + ex2(fmaf(v[u].y, zscale, nm)) + ex2(fmaf(v[u].z, zscale, nm)) +
+             ex2(fmaf(v[u].w, zscale, nm));
+      else
+        s += ex2(fmaf(v[u], zscale, nm));
     }
   };
   if constexpr (UNROLL == 16) {
     // one CTA per SM: two batches of 8, the next one's loads in flight
     // while the current one is summed
-    float4 va[H], vb[H];
+    Unit<VEC> va[H], vb[H];
     int ra[H], rb[H];
     fetch(va, ra);
     while (ra[0] >= 0) {
@@ -254,7 +276,7 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
       consume(vb, rb);
     }
   } else {
-    float4 v[H];
+    Unit<VEC> v[H];
     int vr[H];
     for (;;) {
       fetch(v, vr);
@@ -269,7 +291,7 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
 // UNROLL 16 when the grid has at most one CTA per SM (small batches), where
 // the CTA's bytes in flight set its bandwidth: two batches of 8, one loading
 // while the other is summed.
-template <bool VEC, int UNROLL>
+template <bool VEC, int UNROLL, int HS>
 __global__ void __launch_bounds__(kSampThreads, UNROLL == 8 ? 2 : 1) accept_sampled_kernel(
     const float* __restrict__ tgt, const float* __restrict__ drf, const int32_t* __restrict__ draft,
     const float* __restrict__ u_accept, const float* __restrict__ u_sample, float zscale, int gamma, int vocab,
@@ -313,7 +335,7 @@ __global__ void __launch_bounds__(kSampThreads, UNROLL == 8 ? 2 : 1) accept_samp
   __syncthreads();
 
   // ---- phase 1: per-row (m, s) over this CTA's span of warp-aligned units
-  phase1_span<VEC, UNROLL>(tgt, drf, b, gamma, vocab, zscale, c, CL, part);
+  phase1_span<VEC, UNROLL, HS>(tgt, drf, b, gamma, vocab, zscale, c, CL, part);
   // the next kernel may be scheduled once the logits have streamed through
   pdl_launch_next();
   __syncthreads();
@@ -568,7 +590,7 @@ __global__ void __launch_bounds__(kSampThreads, UNROLL == 8 ? 2 : 1) accept_samp
 // (m, s) of every row to pre[b][part][row] (rows outside its span get the
 // empty pair).  accept_sampled_kernel then merges these instead of
 // streaming the logits itself.
-template <bool VEC>
+template <bool VEC, int HS>
 __global__ void __launch_bounds__(kSampThreads, 2) samp_part_kernel(const float* __restrict__ tgt,
                                                                     const float* __restrict__ drf, float zscale,
                                                                     int gamma, int vocab, int parts,
@@ -581,14 +603,10 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_part_kernel(const float*
   for (int i = tid; i < kSampWarps * kSampMaxRows; i += kSampThreads)
     part[i / kSampMaxRows][i % kSampMaxRows] = make_float2(kEmpty, 0.f);
   pdl_wait();
-  // (at once: the grid is one wave, so the waiting CTAs of samp_resid_kernel
-  // only take places that this one's CTAs have left; with that kernel's loads
-  // issued ahead, 8 sequences of 9 rows of 151936 logits 24.9 -> 24.1 us)
-  pdl_launch_next();
   // the arrival count samp_resid_kernel uses for this sequence starts at 0
   if (c == 0 && tid == 0) arrivals[b] = 0u;
   __syncthreads();
-  phase1_span<VEC, 8>(tgt, drf, b, gamma, vocab, zscale, c, parts, part);
+  phase1_span<VEC, 8, HS>(tgt, drf, b, gamma, vocab, zscale, c, parts, part);
   __syncthreads();
   for (int r = tid; r < rows; r += kSampThreads) {
     float m = kEmpty, s = 0.f;
@@ -596,6 +614,9 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_part_kernel(const float*
     for (int w = 0; w < kSampWarps; ++w) ms_merge(m, s, part[w][r].x, part[w][r].y);
     pre[(static_cast<size_t>(b) * parts + c) * rows + r] = make_float2(m, s);
   }
+  // (at the start it made the call up to 1 us slower: 4 sequences of 17 rows of
+  // 50004 logits 12.9 -> 14.0, 2 of 65 rows of 151936 23.9 -> 25.5)
+  pdl_launch_next();
 }
 
 // Row a's weights at one unit of 4 columns (1 in the scalar layout, the
@@ -771,8 +792,10 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   __threadfence();
   // ---- the last CTA of the sequence: which span holds the threshold
   if (warp == 0) {
-    // the other CTAs' sums, read past L1 (they were written by other SMs);
-    // the first two a lane stay in registers for the scan below
+    // the other CTAs' sums, read past L1 (they were written by other SMs); the
+    // first two a lane stay in registers for the scan below (with u_sample and
+    // the span's units loaded once and ahead: 8 sequences of 17 rows of 151936
+    // logits 24.4 -> 23.5 us, one of 9 rows 12.3 -> 11.3)
     const float2* vs = sums + static_cast<size_t>(b) * rparts;
     const float2 v0 = lane < rparts ? __ldcg(vs + lane) : make_float2(0.f, 0.f);
     const float2 v1 = lane + 32 < rparts ? __ldcg(vs + lane + 32) : make_float2(0.f, 0.f);
@@ -844,20 +867,22 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   const int u0 = min(W, owner_sh * per), u1 = min(W, u0 + per);
   const int k = (u1 - u0 + kSampThreads - 1) / kSampThreads;
   const int t0 = min(u1, u0 + tid * k), t1 = min(u1, t0 + k);
-  // (the weights of the first two stay in registers for the walk: a span is at
-  // most 1024 units, two a thread, unless there are few parts)
+  // (16-byte units: the weights of the first two stay in registers for the
+  // walk; a span is at most 1024 units, two a thread, unless there are few parts)
   const float4 kZero = make_float4(0.f, 0.f, 0.f, 0.f);
   float4 w0 = kZero, w1 = kZero;
-  if (t0 < t1) {
+  if (VEC && t0 < t1) {
     const int second = min(t0 + 1, t1 - 1);
     const UnitW x0 = unit_weights<VEC>(rw, t0), x1 = unit_weights<VEC>(rw, second);
     w0 = mode == 0 ? x0.r : x0.t;
     if (t0 + 1 < t1) w1 = mode == 0 ? x1.r : x1.t;
   }
   float mine = 0.f;
-  mine += (w0.x + w0.y) + (w0.z + w0.w);
-  mine += (w1.x + w1.y) + (w1.z + w1.w);
-  for (int u = t0 + 2; u < t1; ++u) {
+  if (VEC) {
+    mine += (w0.x + w0.y) + (w0.z + w0.w);
+    mine += (w1.x + w1.y) + (w1.z + w1.w);
+  }
+  for (int u = VEC ? t0 + 2 : t0; u < t1; ++u) {
     const UnitW uw = unit_weights<VEC>(rw, u);
     const float4 w = mode == 0 ? uw.r : uw.t;
     mine += (w.x + w.y) + (w.z + w.w);
@@ -886,7 +911,7 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   };
   for (int u = t0; u < t1 && hit < 0; ++u) {
     float4 w = u == t0 ? w0 : w1;
-    if (u > t0 + 1) {
+    if (!VEC || u > t0 + 1) {
       const UnitW uw = unit_weights<VEC>(rw, u);
       w = mode == 0 ? uw.r : uw.t;
     }
@@ -908,9 +933,9 @@ struct SampCapacity {
   int resident16[kSampMaxCluster + 1] = {};  // UNROLL 16
 };
 
-template <bool VEC, int UNROLL>
+template <bool VEC, int UNROLL, int HS>
 cudaError_t max_clusters(int cl, int* n) {
-  auto kern = accept_sampled_kernel<VEC, UNROLL>;
+  auto kern = accept_sampled_kernel<VEC, UNROLL, HS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -928,11 +953,13 @@ cudaError_t max_clusters(int cl, int* n) {
 
 template <int UNROLL>
 cudaError_t min_clusters(int cl, int* n) {
-  int n1 = 0, n2 = 0;
-  cudaError_t e = max_clusters<true, UNROLL>(cl, &n1);
+  int n1 = 0, n2 = 0, n3 = 0;
+  cudaError_t e = max_clusters<true, UNROLL, 8>(cl, &n1);
   if (e != cudaSuccess) return e;
-  e = max_clusters<false, UNROLL>(cl, &n2);
-  *n = n1 < n2 ? n1 : n2;
+  e = max_clusters<false, UNROLL, 8>(cl, &n2);
+  if (e != cudaSuccess) return e;
+  e = max_clusters<false, UNROLL, 16>(cl, &n3);
+  *n = std::min({n1, n2, n3});
   return e;
 }
 
@@ -958,11 +985,21 @@ cudaError_t samp_capacity(const SampCapacity** out) {
   return cudaSuccess;
 }
 
-template <bool VEC, int UNROLL>
+// Scalar units are loaded 16 at a time where a thread has at least five rounds
+// of them (8 sequences of 33 rows of 151935 logits, 244 a thread: 60.4 -> 52.8
+// us; 17 rows of 100001, 87 a thread: 30.6 -> 28.7).  Each row change and the
+// span's end take the slow path for a whole round, so short spans keep 8 (25
+// rows of 50001, 64 a thread: 23.6 us with 8, 24.3 with 16; 20 sequences of 9
+// rows of 1001: 11.7, 13.3).
+bool scalar_rounds(int gamma, int vocab, int ctas) {
+  return (2LL * gamma + 1) * vocab >= 80LL * kSampThreads * ctas;
+}
+
+template <bool VEC, int UNROLL, int HS>
 cudaError_t launch_samp(dim3 grid, unsigned CL, cudaStream_t stream, const float* tl, const float* dl,
                         const int32_t* draft, const float* ua, const float* us, float zscale, int gamma, int vocab,
                         int32_t* accepted_len, int32_t* out_tokens, int32_t* err_word) {
-  return launch_overlapped(accept_sampled_kernel<VEC, UNROLL>, grid, dim3(kSampThreads), 0, stream, CL, tl, dl,
+  return launch_overlapped(accept_sampled_kernel<VEC, UNROLL, HS>, grid, dim3(kSampThreads), 0, stream, CL, tl, dl,
                            draft, ua, us, zscale, gamma, vocab, accepted_len, out_tokens, err_word);
 }
 
@@ -1018,10 +1055,11 @@ cudaError_t launch_accept_sampled(const float* target_logits, const float* draft
     const dim3 pgrid(static_cast<unsigned>(n));
     const int rparts = samp_resid_parts(parts, vocab);
     const dim3 rgrid(static_cast<unsigned>(Bt) * rparts);
-    cudaError_t e = vec4 ? launch_overlapped(samp_part_kernel<true>, pgrid, dim3(kSampThreads), 0, stream, 1u,
-                                             target_logits, draft_logits, zscale, gamma, vocab, parts, pre, arrivals)
-                         : launch_overlapped(samp_part_kernel<false>, pgrid, dim3(kSampThreads), 0, stream, 1u,
-                                             target_logits, draft_logits, zscale, gamma, vocab, parts, pre, arrivals);
+    auto part_kernel = vec4                                 ? samp_part_kernel<true, 8>
+                       : scalar_rounds(gamma, vocab, parts) ? samp_part_kernel<false, 16>
+                                                            : samp_part_kernel<false, 8>;
+    cudaError_t e = launch_overlapped(part_kernel, pgrid, dim3(kSampThreads), 0, stream, 1u, target_logits,
+                                      draft_logits, zscale, gamma, vocab, parts, pre, arrivals);
     if (e != cudaSuccess) return e;
     return vec4 ? launch_overlapped(samp_resid_kernel<true>, rgrid, dim3(kSampThreads), 0, stream, 1u, target_logits,
                                     draft_logits, draft, u_accept, u_sample, zscale, gamma, vocab, accepted_len,
@@ -1046,15 +1084,12 @@ cudaError_t launch_accept_sampled(const float* target_logits, const float* draft
   const bool deep = cap->resident16[CL] >= Bt;
   const dim3 grid(static_cast<unsigned>(Bt) * CL);
   const unsigned ucl = static_cast<unsigned>(CL);
-  if (vec4)
-    return deep ? launch_samp<true, 16>(grid, ucl, stream, target_logits, draft_logits, draft, u_accept, u_sample,
-                                        zscale, gamma, vocab, accepted_len, out_tokens, err_word)
-                : launch_samp<true, 8>(grid, ucl, stream, target_logits, draft_logits, draft, u_accept, u_sample,
-                                       zscale, gamma, vocab, accepted_len, out_tokens, err_word);
-  return deep ? launch_samp<false, 16>(grid, ucl, stream, target_logits, draft_logits, draft, u_accept, u_sample,
-                                       zscale, gamma, vocab, accepted_len, out_tokens, err_word)
-              : launch_samp<false, 8>(grid, ucl, stream, target_logits, draft_logits, draft, u_accept, u_sample,
-                                      zscale, gamma, vocab, accepted_len, out_tokens, err_word);
+  const bool many = scalar_rounds(gamma, vocab, CL);
+  auto launch = vec4 ? (deep ? launch_samp<true, 16, 8> : launch_samp<true, 8, 8>)
+                : many ? (deep ? launch_samp<false, 16, 16> : launch_samp<false, 8, 16>)
+                       : (deep ? launch_samp<false, 16, 8> : launch_samp<false, 8, 8>);
+  return launch(grid, ucl, stream, target_logits, draft_logits, draft, u_accept, u_sample, zscale, gamma, vocab,
+                accepted_len, out_tokens, err_word);
 }
 
 }  // namespace simsd
