@@ -1,7 +1,7 @@
-"""Stochastic acceptance over rows that start off the 16-byte grid: 16-byte
-pieces that cover a row, its first and last holding neighbours' values.  Every
+"""Stochastic acceptance over rows that start off the 16-byte grid.  Every
 vocabulary remainder and base shift, with values around the rows that would
-change the sums or the draw if they were read; decisions and tokens by the
+change the sums or the draw if they were read, spans on both sides of the line
+between 8 and 16 scalar loads at a time; decisions and tokens by the
 oracle outside the fp32 band, as in test_gpu_accept_sampled.py, through the
 cluster kernel and the split one."""
 import dataclasses
@@ -24,7 +24,7 @@ def _shifted(t, shift):
 
 @pytest.mark.parametrize("shift", [0, 1, 2, 3])
 @pytest.mark.parametrize("Bt,gamma,V", [(3, 2, 5), (2, 3, 127), (6, 4, 30001), (2, 8, 50002), (1, 16, 50003),
-                                        (3, 4, 1024), (2, 1, 2)])
+                                        (3, 4, 1024), (2, 1, 2), (8, 20, 50001), (24, 4, 65537)])
 def test_row_ends(monkeypatch, Bt, gamma, V, shift):
     si = inputs.make_sampled_inputs(Bt, gamma, V, seed=V + shift, device="cuda")
     # heavy first and last columns: drafts and draws fall on the rows' ends
