@@ -451,8 +451,13 @@ __global__ void __maxnreg__(kMaxRegs)
           s_issued = true;
         }
         tc_commit(smem_u32(&sm.bar_empty[st]));
-        tc_commit(smem_u32(&sm.bar_pv));
       }
+      // The epilogue's barrier, committed once, behind the last PV.  (One
+      // phase a tile would leave its wait ambiguous: S of the last tile is
+      // handed over ahead of the commits of the PV before it, so a parity test
+      // could find that PV's phase still open and take an older one for its
+      // own.)
+      if (ok) tc_commit(smem_u32(&sm.bar_pv));
       if (!ok) signal_abort(sm, p.err_word);
       // every MMA issued by this thread has completed once this fires
       tc_commit(smem_u32(&sm.bar_drain));
@@ -655,9 +660,9 @@ __global__ void __maxnreg__(kMaxRegs)
     // the next layer's set-up then runs under it (36 layers of 8 sequences,
     // 809 us with the trigger at exit, 768 here)
     pdl_launch_next();
-    // ---- epilogue: O of the last PV, scaled by 1/l
-    const bool have_o =
-        ok && ntiles > 0 && mbar_wait_warp(smem_u32(&sm.bar_pv), (ntiles - 1) & 1, abort_flag, p.wait_ns);
+    // ---- epilogue: O of the last PV, scaled by 1/l (bar_pv has one phase: it
+    // completes when every MMA of the CTA has)
+    const bool have_o = ok && ntiles > 0 && mbar_wait_warp(smem_u32(&sm.bar_pv), 0, abort_flag, p.wait_ns);
     if (have_o) tc_fence_after();
     const bool any = have_o && active && l_sum > 0.f;
     const int h = kvh * p.g + hl;
