@@ -114,12 +114,14 @@ __global__ void __maxnreg__(kF32Regs)
   pdl_wait();
   pdl_launch_next();
   const int S = 2 * a.gamma, g = a.Hq / a.Hkv, R = S * g;
-  // grid: (sequence, row block, split) x KV head; the splits of a unit are
-  // adjacent (a cluster), then its row blocks (which share its K/V in L2)
+  // grid: KV head, then sequence, row block, split (one dimension: the second
+  // ends at 65535); the splits of a unit are adjacent (a cluster), then its
+  // row blocks (which share its K/V in L2)
   const unsigned bx = blockIdx.x / static_cast<unsigned>(nsplit);
   const int split = blockIdx.x - bx * nsplit;
-  const int b = bx / static_cast<unsigned>(rb), rblk = bx - b * rb;
-  const int kvh = blockIdx.y;
+  const unsigned u = bx / static_cast<unsigned>(rb);
+  const int rblk = bx - u * rb;
+  const int kvh = u / static_cast<unsigned>(a.Bt), b = u - kvh * a.Bt;
   const int blk_row0 = rblk * W * kF32Rows;    // the CTA's first row of the unit
   const int row0 = blk_row0 + warp * kF32Rows;  // this warp's
 
@@ -667,7 +669,7 @@ cudaError_t launch(const AttnF32Args& a, cudaStream_t stream) {
   }
   ns = std::max(ns, 1);
   const size_t smem = ns > 1 ? smem_for<D>(W, k) : F32Layout<D>::bytes(W);
-  return launch_overlapped(attention_f32_kernel<D>, dim3(static_cast<unsigned>(a.Bt) * rb * ns, a.Hkv),
+  return launch_overlapped(attention_f32_kernel<D>, dim3(static_cast<unsigned>(units * ns)),
                            dim3(32 * (W + 1)), smem, stream, static_cast<unsigned>(ns), a, rb, ns);
 }
 
