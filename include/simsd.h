@@ -368,7 +368,7 @@ SIMSD_API int simsd_plan_accept(int sampled, int Bt, int gamma, int vocab, int n
 
 /*
  * simsd_debug_expire_next_wait -- test hook for failure detection; the paper
- * has no counterpart.  Arms the next bf16 simsd_verify_attention
+ * has no counterpart.  Arms the next simsd_verify_attention
  * (which = SIMSD_DEBUG_WAIT_ATTENTION) or simsd_accept
  * (which = SIMSD_DEBUG_WAIT_ACCEPT) call made by this host thread so that
  * one of its on-device barriers expects one arrival more than ever comes
@@ -376,11 +376,14 @@ SIMSD_API int simsd_plan_accept(int sampled, int Bt, int gamma, int vocab, int n
  * 1 s.  The wait then runs out: the kernel sets SIMSD_EW_TIMEOUT, stops
  * every warp, waits (with the full limit) for its own copies and MMAs in
  * flight, frees its tensor memory and returns; the outputs of that call are
- * undefined and the context stays usable.  Attention: the softmax warps'
- * hand-off of P to the MMA issuer.  Acceptance: CTA 0's wait for the
- * per-CTA row maxima; armed only where every sequence runs as a single CTA
- * (a batch too large for one cluster per sequence to be resident), else the
- * call returns SIMSD_ERR_UNSUPPORTED.  The arm is consumed by that call.
+ * undefined and the context stays usable.  Attention, bf16: the softmax warps'
+ * hand-off of P to the MMA issuer.  Attention, fp32: the release of a K tile
+ * to the producer, which waits for it where a CTA takes more than one tile
+ * of 32 keys (calls of shorter prefixes complete normally).  Acceptance:
+ * CTA 0's wait for the per-CTA row maxima; armed only where every sequence
+ * runs as a single CTA (a batch too large for one cluster per sequence to be
+ * resident), else the call returns SIMSD_ERR_UNSUPPORTED.  The arm is consumed
+ * by that call.
  */
 #define SIMSD_DEBUG_WAIT_ATTENTION 1
 #define SIMSD_DEBUG_WAIT_ACCEPT 2

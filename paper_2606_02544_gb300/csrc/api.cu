@@ -152,7 +152,7 @@ int verify_attention_impl(int dtype, const void* q, const void* k_new, const voi
     a.d = d;
     a.num_sms = info.num_sms;
     a.scale = scale;
-    cudaError_t e = simsd::launch_attention_f32(a, s);
+    cudaError_t e = simsd::launch_attention_f32(a, s, fault);
     return e == cudaSuccess ? SIMSD_OK : cuda_fail(e, "attention_f32 launch");
   }
   if (dtype != SIMSD_BF16) return unsupported("dtype");

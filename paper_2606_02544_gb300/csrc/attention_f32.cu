@@ -33,8 +33,9 @@
 // rows and new keys are rotated in shared memory; cached keys are stored
 // rotated.
 //
-// Every mbarrier wait is bounded: one that expires sets SIMSD_EW_TIMEOUT, the
-// CTA leaves its loops, waits for its own copies and finishes (its output is
+// Every mbarrier wait is bounded (a consumer's also ends with the producer's,
+// through the abort flag): one that expires sets SIMSD_EW_TIMEOUT, the CTA
+// leaves its loops, waits for its own copies and finishes (its output is
 // undefined).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -94,6 +95,7 @@ __global__ void __maxnreg__(kF32Regs)
   __shared__ int lab_tau[64], lab_pos[64];
   __shared__ uint8_t lab_sect[64];
   __shared__ int bad_sh, abort_sh;
+  __shared__ int asked[2];  // tiles of K and of V requested
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int W = (blockDim.x >> 5) - 1;  // consumer warps
   const bool producer = warp == W;
@@ -106,7 +108,7 @@ __global__ void __maxnreg__(kF32Regs)
     mbar_init(smem_u32(&bar_q), 1);
     mbar_init(smem_u32(&bar_k), 1);
     mbar_init(smem_u32(&bar_v), 1);
-    mbar_init(smem_u32(&bar_kfree), W);
+    mbar_init(smem_u32(&bar_kfree), a.k_release);
     mbar_init(smem_u32(&bar_vfree), W);
     fence_mbar_init();
   }
@@ -177,16 +179,26 @@ __global__ void __maxnreg__(kF32Regs)
       if (src != 0) bulk_load(smem_u32(dst + lane * KR), (src == 2 ? fresh : cache) + off, kRowBytes, smem_u32(bar));
     };
     bool ok = true;
-    int it = 0;
+    int it = 0, nk = 0, nv = 0;
     for (int t = split; ok && t < T; t += nsplit, ++it) {
       long long off = 0;
       const int src = locate(t, off);
-      ok = it == 0 || mbar_wait_warp(smem_u32(&bar_kfree), (it - 1) & 1, abort_flag);
-      if (ok) load_tile(smem, a.k_cache, a.k_new, &bar_k, off, src);
-      ok = ok && (it == 0 || mbar_wait_warp(smem_u32(&bar_vfree), (it - 1) & 1, abort_flag));
-      if (ok) load_tile(smem + L::kV, a.v_cache, a.v_new, &bar_v, off, src);
+      ok = it == 0 || mbar_wait_warp(smem_u32(&bar_kfree), (it - 1) & 1, abort_flag, a.wait_ns);
+      if (ok) {
+        load_tile(smem, a.k_cache, a.k_new, &bar_k, off, src);
+        ++nk;
+      }
+      ok = ok && (it == 0 || mbar_wait_warp(smem_u32(&bar_vfree), (it - 1) & 1, abort_flag, a.wait_ns));
+      if (ok) {
+        load_tile(smem + L::kV, a.v_cache, a.v_new, &bar_v, off, src);
+        ++nv;
+      }
     }
-    if (!ok && lane == 0) *abort_flag = 1;
+    if (lane == 0) {
+      asked[0] = nk;
+      asked[1] = nv;
+      if (!ok) *abort_flag = 1;
+    }
   } else {
     // slot labels, and every page the sequence needs is checked, while the
     // first loads are in flight
@@ -476,14 +488,14 @@ __global__ void __maxnreg__(kF32Regs)
   __syncthreads();
   if (*abort_flag) {
     // a wait expired: the copies still in flight are waited for (with the
-    // full limit), so that none lands after the CTA has gone
-    if (tid == 0) raise_error(a.err_word, SIMSD_EW_TIMEOUT);
-    if (producer && lane == 0) {
+    // full limit), so that none lands after the CTA has gone.  A tile is
+    // requested after the one before has been consumed, so only the last
+    // phase can be open.
+    if (tid == 0) {
+      raise_error(a.err_word, SIMSD_EW_TIMEOUT);
       mbar_wait(smem_u32(&bar_q), 0, nullptr);
-      for (uint32_t ph = 0; ph < 2; ++ph) {
-        mbar_wait(smem_u32(&bar_k), ph, nullptr);
-        mbar_wait(smem_u32(&bar_v), ph, nullptr);
-      }
+      if (asked[0] > 0) mbar_wait(smem_u32(&bar_k), (asked[0] - 1) & 1, nullptr);
+      if (asked[1] > 0) mbar_wait(smem_u32(&bar_v), (asked[1] - 1) & 1, nullptr);
     }
     __syncthreads();
   }
@@ -638,7 +650,7 @@ cudaError_t resident_clusters(int W, int k, int ns, int* out) {
 }
 
 template <int D>
-cudaError_t launch(const AttnF32Args& a, cudaStream_t stream) {
+cudaError_t launch(AttnF32Args a, cudaStream_t stream, const WaitFault& fault) {
   // row groups of 8, at most eight to a row block, spread evenly over the blocks
   const int groups = (2 * a.gamma * (a.Hq / a.Hkv) + kF32Rows - 1) / kF32Rows;
   const int rb = (groups + kF32MaxWarps - 1) / kF32MaxWarps;
@@ -668,6 +680,8 @@ cudaError_t launch(const AttnF32Args& a, cudaStream_t stream) {
     if (fit >= units) break;
   }
   ns = std::max(ns, 1);
+  a.wait_ns = fault.wait_ns ? fault.wait_ns : kWaitLimitNs;
+  a.k_release = W + fault.extra;
   const size_t smem = ns > 1 ? smem_for<D>(W, k) : F32Layout<D>::bytes(W);
   return launch_overlapped(attention_f32_kernel<D>, dim3(static_cast<unsigned>(units * ns)),
                            dim3(32 * (W + 1)), smem, stream, static_cast<unsigned>(ns), a, rb, ns);
@@ -675,8 +689,8 @@ cudaError_t launch(const AttnF32Args& a, cudaStream_t stream) {
 
 }  // namespace
 
-cudaError_t launch_attention_f32(const AttnF32Args& a, cudaStream_t stream) {
-  return a.d == 64 ? launch<64>(a, stream) : launch<128>(a, stream);
+cudaError_t launch_attention_f32(const AttnF32Args& a, cudaStream_t stream, const WaitFault& fault) {
+  return a.d == 64 ? launch<64>(a, stream, fault) : launch<128>(a, stream, fault);
 }
 
 }  // namespace simsd

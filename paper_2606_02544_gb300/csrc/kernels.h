@@ -69,8 +69,12 @@ struct AttnF32Args {
   int32_t* err_word;
   int num_pages, max_pages, page_size, Bt, gamma, Hq, Hkv, d, num_sms;
   float scale;
+  // set at launch: the limit of the producer's waits, and the arrivals that
+  // release a K tile (one a consumer warp; one more makes the wait run out)
+  unsigned long long wait_ns;
+  uint32_t k_release;
 };
-cudaError_t launch_attention_f32(const AttnF32Args& a, cudaStream_t stream);
+cudaError_t launch_attention_f32(const AttnF32Args& a, cudaStream_t stream, const WaitFault& fault = WaitFault{});
 
 // bf16 tensor-core path
 struct AttnTcPlan {
