@@ -88,6 +88,13 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gmem) : "memory");
 }
 
+// Two floats that another SM may have written: a strong load, kept in order
+// with the fences around it.
+__device__ __forceinline__ float2 ld_gpu_f32x2(const float2* p) {
+  float2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Row `row` of the combined row space: target rows 0..gamma, then draft rows.
@@ -792,16 +799,17 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
   __threadfence();
   // ---- the last CTA of the sequence: which span holds the threshold
   if (warp == 0) {
-    // the other CTAs' sums, read past L1 (they were written by other SMs); the
+    // the other CTAs' sums, written by other SMs: loads that the fence above
+    // orders behind the arrival count (a plain cached load may be moved); the
     // first two a lane stay in registers for the scan below (with u_sample and
     // the span's units loaded once and ahead: 8 sequences of 17 rows of 151936
     // logits 24.4 -> 23.5 us, one of 9 rows 12.3 -> 11.3)
     const float2* vs = sums + static_cast<size_t>(b) * rparts;
-    const float2 v0 = lane < rparts ? __ldcg(vs + lane) : make_float2(0.f, 0.f);
-    const float2 v1 = lane + 32 < rparts ? __ldcg(vs + lane + 32) : make_float2(0.f, 0.f);
+    const float2 v0 = lane < rparts ? ld_gpu_f32x2(vs + lane) : make_float2(0.f, 0.f);
+    const float2 v1 = lane + 32 < rparts ? ld_gpu_f32x2(vs + lane + 32) : make_float2(0.f, 0.f);
     float tr = v0.x + v1.x, tt = v0.y + v1.y;
     for (int q = lane + 64; q < rparts; q += 32) {
-      const float2 v = __ldcg(vs + q);
+      const float2 v = ld_gpu_f32x2(vs + q);
       tr += v.x;
       tt += v.y;
     }
@@ -821,7 +829,7 @@ __global__ void __launch_bounds__(kSampThreads, 2) samp_resid_kernel(
       const int q = q0 + lane;
       const float2 vq = q0 == 0    ? v0
                         : q0 == 32 ? v1
-                                   : (q < rparts ? __ldcg(vs + q) : make_float2(0.f, 0.f));
+                                   : (q < rparts ? ld_gpu_f32x2(vs + q) : make_float2(0.f, 0.f));
       const float wq = mode == 0 ? vq.x : vq.y;
       float incl = wq;
 #pragma unroll
