@@ -424,11 +424,20 @@ __global__ void __maxnreg__(kF32Regs)
     // see: a tile with such a value among its new slots takes the select below
     bool odd = false;
     if (has_new) {
-      for (int j = max(0, n - t * kF32Keys); j < kF32Keys; ++j) {
-        float v[NC];
-        load_v(j, v);
+      // (eight rows at a time, cached keys before the first slot among them:
+      // the select is right for those too.  One row after the other to the
+      // tile's end took 1900 cycles of a call of one tile a CTA; a step of one
+      // sequence of 128 keys 15.7 -> 14.8 us.)
+      const int j1 = min(kF32Keys, nkeys - t * kF32Keys);
+#pragma unroll 1
+      for (int j0 = max(0, n - t * kF32Keys) & ~7; j0 < j1; j0 += 8) {
 #pragma unroll
-        for (int c = 0; c < NC; ++c) odd |= !(fabsf(v[c]) < INFINITY);
+        for (int j = 0; j < 8; ++j) {
+          float v[NC];
+          load_v(j0 + j, v);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) odd |= !(fabsf(v[c]) < INFINITY);
+        }
       }
     }
     if (!__any_sync(full, odd)) {
