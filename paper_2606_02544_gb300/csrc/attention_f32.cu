@@ -58,6 +58,7 @@ constexpr int kF32Keys = 32;     // keys of a tile
 constexpr int kF32MaxWarps = 8;  // row groups of a row block (then the producer warp)
 constexpr int kF32MaxSplit = 16;  // key ranges of a unit (cluster size)
 constexpr int kF32Merge = 4;     // ranges merged at a time
+constexpr int kF32GridY = 65535;  // most blocks of a grid in y
 constexpr int kF32Regs = 112;    // 18 warps an SM by the register file
 // shared memory: of an SM, of one CTA (dynamic), and of a CTA beside its
 // dynamic part (static and reserved, rounded up)
@@ -102,6 +103,10 @@ __global__ void __maxnreg__(kF32Regs)
   const int half = lane >> 4, kp = lane & 15;
   const unsigned full = 0xffffffffu;
   volatile int* abort_flag = &abort_sh;
+  // KV heads lie over y and z, each of which ends at 65535 (in x the divisions
+  // that find one cost 0.2 us a call); the last z may not be full
+  const int kvh = blockIdx.z * kF32GridY + blockIdx.y;
+  if (kvh >= a.Hkv) return;  // (a whole cluster)
   if (tid == 0) {
     bad_sh = 0;
     abort_sh = 0;
@@ -116,14 +121,11 @@ __global__ void __maxnreg__(kF32Regs)
   pdl_wait();
   pdl_launch_next();
   const int S = 2 * a.gamma, g = a.Hq / a.Hkv, R = S * g;
-  // grid: KV head, then sequence, row block, split (one dimension: the second
-  // ends at 65535); the splits of a unit are adjacent (a cluster), then its
-  // row blocks (which share its K/V in L2)
+  // grid: (sequence, row block, split) x KV head; the splits of a unit are
+  // adjacent (a cluster), then its row blocks (which share its K/V in L2)
   const unsigned bx = blockIdx.x / static_cast<unsigned>(nsplit);
   const int split = blockIdx.x - bx * nsplit;
-  const unsigned u = bx / static_cast<unsigned>(rb);
-  const int rblk = bx - u * rb;
-  const int kvh = u / static_cast<unsigned>(a.Bt), b = u - kvh * a.Bt;
+  const int b = bx / static_cast<unsigned>(rb), rblk = bx - b * rb;
   const int blk_row0 = rblk * W * kF32Rows;    // the CTA's first row of the unit
   const int row0 = blk_row0 + warp * kF32Rows;  // this warp's
 
@@ -691,8 +693,9 @@ cudaError_t launch(AttnF32Args a, cudaStream_t stream, const WaitFault& fault) {
   ns = std::max(ns, 1);
   a.wait_ns = fault.wait_ns ? fault.wait_ns : kWaitLimitNs;
   a.k_release = W + fault.extra;
+  const unsigned hy = std::min(a.Hkv, kF32GridY), hz = (static_cast<unsigned>(a.Hkv) + kF32GridY - 1) / kF32GridY;
   const size_t smem = ns > 1 ? smem_for<D>(W, k) : F32Layout<D>::bytes(W);
-  return launch_overlapped(attention_f32_kernel<D>, dim3(static_cast<unsigned>(units * ns)),
+  return launch_overlapped(attention_f32_kernel<D>, dim3(static_cast<unsigned>(a.Bt) * rb * ns, hy, hz),
                            dim3(32 * (W + 1)), smem, stream, static_cast<unsigned>(ns), a, rb, ns);
 }
 
