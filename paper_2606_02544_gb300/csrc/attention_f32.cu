@@ -91,8 +91,10 @@ __global__ void __maxnreg__(kF32Regs)
   constexpr int NC = D / 32;  // columns of a lane in O
   constexpr int KR = L::kRow;
   constexpr uint32_t kRowBytes = D * sizeof(float);
+  constexpr int kChunks = D / 4;          // 16-byte pieces of a row
+  constexpr int kPerCopy = 32 / kChunks;  // rows a warp's copy covers, a piece a lane
   extern __shared__ __align__(16) float smem[];
-  __shared__ __align__(8) uint64_t bar_q, bar_k, bar_v, bar_kfree, bar_vfree;
+  __shared__ __align__(8) uint64_t bar_k, bar_v, bar_kfree, bar_vfree;
   __shared__ int lab_tau[64], lab_pos[64];
   __shared__ uint8_t lab_sect[64];
   __shared__ int bad_sh, abort_sh;
@@ -110,7 +112,6 @@ __global__ void __maxnreg__(kF32Regs)
   if (tid == 0) {
     bad_sh = 0;
     abort_sh = 0;
-    mbar_init(smem_u32(&bar_q), 1);
     mbar_init(smem_u32(&bar_k), 1);
     mbar_init(smem_u32(&bar_v), 1);
     mbar_init(smem_u32(&bar_kfree), a.k_release);
@@ -144,11 +145,6 @@ __global__ void __maxnreg__(kF32Regs)
     // loaded beside it (and not used past it)
     const int pi0 = (split * kF32Keys + lane) / a.page_size;
     const int page0 = pi0 < a.max_pages ? bt[pi0] : -1;
-    const int rows = min(R - blk_row0, W * kF32Rows);  // at least 1
-    if (lane == 0) mbar_arrive_expect_tx(smem_u32(&bar_q), static_cast<uint32_t>(rows) * kRowBytes);
-    __syncwarp();
-    for (int i = lane; i < rows; i += 32)
-      bulk_load(smem_u32(smem + L::kQ + i * KR), a.q + q_offset(blk_row0 + i), kRowBytes, smem_u32(&bar_q));
     // keys 0..n-1 are the prefix rows, keys n..n+S-1 the new slots; lane i finds
     // key i of a tile.  Slots of padding are no row's key: their rows are zeros,
     // as are rows past the last key and pages out of range.  src: 1 cache, 2 new
@@ -202,6 +198,22 @@ __global__ void __maxnreg__(kF32Regs)
       if (!ok) *abort_flag = 1;
     }
   } else {
+    // this warp's query rows (zeros past the unit's last), waited for below.
+    // The producer's bulk copies, one a row and 58 cycles each to issue, held
+    // up the first K: 128 rows of d 64 over 24 keys 9.9 -> 8.3 us a call, 8
+    // sequences of 64 rows a KV head over 128 keys 21.3 -> 19.6.
+    {
+      float* qs = smem + L::kQ + warp * kF32Rows * KR;
+      const int own = min(row0 + (lane & (kF32Rows - 1)), R - 1);
+      const unsigned long long from = reinterpret_cast<unsigned long long>(a.q + q_offset(own));
+      const int sub = lane / kChunks, col = 4 * (lane % kChunks);
+#pragma unroll
+      for (int i = 0; i < kF32Rows; i += kPerCopy) {
+        const int r = i + sub;
+        const float* row = reinterpret_cast<const float*>(__shfl_sync(full, from, r));
+        cp_async16(smem_u32(qs + r * KR + col), row + col, row0 + r < R ? 16u : 0u);
+      }
+    }
     // slot labels, and every page the sequence needs is checked, while the
     // first loads are in flight
     const int nt = 32 * W;
@@ -251,13 +263,10 @@ __global__ void __maxnreg__(kF32Regs)
   const bool act = lane < kF32Rows && own_row < R && !seq_bad && lab_sect[min(own_slot, S - 1)] != kSectPad;
   if (!act) vis = 0ull;
   act_rows = __ballot_sync(full, act);
-  bool ok = mbar_wait_warp(smem_u32(&bar_q), 0, abort_flag);
-  if (row0 + kF32Rows > R) {
-    // rows past the unit: any finite value
-    for (int i = max(0, R - row0); i < kF32Rows; ++i)
-      for (int c = lane; c < D; c += 32) qs[i * KR + c] = 0.f;
-  }
-  if (a.rope_pos && ok) {
+  bool ok = true;
+  cp_async_wait_all();
+  __syncwarp();
+  if (a.rope_pos) {
     // lane i turns pairs i, i + 32, ...; rows of one slot share the angles
     float sn[D / 64], cs[D / 64];
     int prev = -1;
@@ -504,7 +513,6 @@ __global__ void __maxnreg__(kF32Regs)
     // phase can be open.
     if (tid == 0) {
       raise_error(a.err_word, SIMSD_EW_TIMEOUT);
-      mbar_wait(smem_u32(&bar_q), 0, nullptr);
       if (asked[0] > 0) mbar_wait(smem_u32(&bar_k), (asked[0] - 1) & 1, nullptr);
       if (asked[1] > 0) mbar_wait(smem_u32(&bar_v), (asked[1] - 1) & 1, nullptr);
     }
