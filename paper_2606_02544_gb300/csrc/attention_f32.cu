@@ -120,7 +120,6 @@ __global__ void __maxnreg__(kF32Regs)
   }
   __syncthreads();
   pdl_wait();
-  pdl_launch_next();
   const int S = 2 * a.gamma, g = a.Hq / a.Hkv, R = S * g;
   // grid: (sequence, row block, split) x KV head; the splits of a unit are
   // adjacent (a cluster), then its row blocks (which share its K/V in L2)
@@ -505,6 +504,7 @@ __global__ void __maxnreg__(kF32Regs)
     if (!((act_rows >> row_of(half, i)) & 1u)) l[i] = 0.f;
   }
   }  // consumer warps
+  pdl_launch_next();  // (the tiles are done: common.cuh)
   __syncthreads();
   if (*abort_flag) {
     // a wait expired: the copies still in flight are waited for (with the
