@@ -89,6 +89,19 @@ def _traffic(workload, kernel):
         return None
 
 
+def _attention_kernel(wl, si):
+    """The kernel (and merge launch) one attention call of the workload runs."""
+    import torch
+
+    from paper_2606_02544_gb300 import simsd
+    p = simsd.simsd_plan_attention(simsd.SIMSD_F32 if wl.dtype == "f32" else simsd.SIMSD_BF16, wl.Bt, wl.gamma, wl.Hq,
+                                   wl.Hkv, wl.d, si.block_table.shape[1], wl.page_size,
+                                   torch.cuda.get_device_properties(0).multi_processor_count)
+    name = {1: "attention_tc256_kernel", 2: "attention_f32_kernel"}.get(
+        p["kernel"], "attention_tc64_kernel" if p["rows_blk"] <= 64 else "attention_tc_kernel")
+    return name + (" + merge launch" if p["ws_bytes"] else "")
+
+
 def workload_config(wl, layers):
     """The workload description both arms print in ``config``."""
     return {"workload": wl.name, "Bt": wl.Bt, "Hq": wl.Hq, "Hkv": wl.Hkv, "head_dim": wl.d, "gamma": wl.gamma,
@@ -291,7 +304,7 @@ def run_gpu(args):
     acc_launch_ms = statistics.median(acc_times)
     attn_gbs = attn_bytes / (attn_launch_ms * 1e-3) / 1e9
     acc_gbs = acc_bytes / (acc_launch_ms * 1e-3) / 1e9
-    attn_roof = {"kernel": "simsd_verify_attention (attention_tc_kernel + combine_kernel when split)", "bound": "hbm",
+    attn_roof = {"kernel": f"simsd_verify_attention ({_attention_kernel(wl, si)})", "bound": "hbm",
                  "achieved": round(attn_gbs, 1), "peak": hbm_peak, "unit": "GB/s",
                  "frac": round(attn_gbs / hbm_peak, 4), "frac_of_8TBs": round(attn_gbs / 8000.0, 4),
                  "peak_source": peak_kind, "algorithmic_bytes_per_launch": int(attn_bytes),

@@ -136,8 +136,8 @@ __device__ __forceinline__ void scan_span_vec(const float* __restrict__ base, in
 // and the start of the next (its values are then seen one by one), and the
 // first and the last unit may reach past the block (their values inside it
 // are loaded one by one).  Against one 4-byte load at a time, which this
-// replaced, 16 sequences of 9 rows of 50001 logits: 20.0 -> 10.9 us (the
-// host's calls by then); 64 sequences 69.7 -> 27.7 us.
+// replaced, call after call in a graph: 16 sequences of 9 rows of 50001 logits
+// 13.5 -> 10.4 us, 64 sequences 68.0 -> 26.7.
 template <int UNROLL>
 __device__ __forceinline__ void scan_span_any(const float* __restrict__ base, int rows, int vocab, int c, int CL,
                                               unsigned long long* best) {
@@ -520,10 +520,13 @@ cudaError_t launch_accept(const float* logits, const int32_t* draft, int Bt, int
   // first): 38 sequences 41.6 -> 34.9 us, 36 36.6 -> 32.4, 30 35.7 -> 28.7, 28
   // 30.0 -> 26.8, 23 25.4 -> 22.9, 19 22.6 -> 20.2, one sequence fewer in each
   // case 37.8 -> 34.5, 33.0 -> 31.8, 32.2 -> 28.3, 26.6 -> 26.0, 22.9 -> 22.2, 20.1
-  // -> 19.7; two fewer 1 to 4% slower, hence the line.  A call that is waited
-  // for takes 0 to 1.7 us more.  Clusters of up to 6 gain less than such a
-  // call loses (96 sequences, 3 -> 2: 95.4 -> 89.2 and 92.9 -> 106.5 us) or
-  // nothing, those of 16 nothing.
+  // -> 19.7; two fewer 1 to 4% slower, hence the line.  Between attention and
+  // commit in captured steps (four or five shapes a batch, 5 to 17 rows of
+  // 151936 or 32000 logits) a step takes 0.91 and 0.90 of its time at 19 and 18
+  // sequences and 0.98 to 1.02 on average at the others (0.93 to 1.10 in single
+  // shapes); a call that is waited for takes 0 to 2.2 us more.  Clusters of up
+  // to 6 gain less than such a call loses (96 sequences, 3 -> 2: 95.4 -> 89.2
+  // and 92.9 -> 106.5 us) or nothing, those of 16 nothing.
   if (CL >= 7 && CL < kMaxCluster && cap->resident[CL] - Bt < 2) --CL;
   if (fault.extra && CL > 1) return cudaErrorNotSupported;
   return launch_overlapped(vec4 ? accept_kernel<8, true> : accept_kernel<8, false>,

@@ -270,7 +270,7 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
     }
   };
   if constexpr (UNROLL == 16) {
-    // one CTA per SM: two batches of 8, the next one's loads in flight
+    // one CTA per SM: two batches of H units, the next one's loads in flight
     // while the current one is summed
     Unit<VEC> va[H], vb[H];
     int ra[H], rb[H];
@@ -296,8 +296,8 @@ __device__ __forceinline__ void phase1_span(const float* __restrict__ tgt, const
 
 // Units in flight per thread in phase 1: UNROLL 8 with two CTAs per SM;
 // UNROLL 16 when the grid has at most one CTA per SM (small batches), where
-// the CTA's bytes in flight set its bandwidth: two batches of 8, one loading
-// while the other is summed.
+// the CTA's bytes in flight set its bandwidth: two batches (of 8 units, or of
+// HS scalar ones), one loading while the other is summed.
 template <bool VEC, int UNROLL, int HS>
 __global__ void __launch_bounds__(kSampThreads, UNROLL == 8 ? 2 : 1) accept_sampled_kernel(
     const float* __restrict__ tgt, const float* __restrict__ drf, const int32_t* __restrict__ draft,
@@ -994,7 +994,7 @@ cudaError_t samp_capacity(const SampCapacity** out) {
 }
 
 // Scalar units are loaded 16 at a time where a thread has at least five rounds
-// of them (8 sequences of 33 rows of 151935 logits, 244 a thread: 60.4 -> 52.8
+// of them (8 sequences of 33 rows of 151935 logits, 258 a thread: 60.4 -> 52.8
 // us; 17 rows of 100001, 87 a thread: 30.6 -> 28.7).  Each row change and the
 // span's end take the slow path for a whole round, so short spans keep 8 (25
 // rows of 50001, 64 a thread: 23.6 us with 8, 24.3 with 16; 20 sequences of 9
@@ -1014,8 +1014,8 @@ cudaError_t launch_samp(dim3 grid, unsigned CL, cudaStream_t stream, const float
 }  // namespace
 
 int samp_parts(int Bt, int gamma, int vocab, int num_sms) {
-  // as for greedy acceptance: few sequences, each with at least 6 MiB of
-  // logits (target and draft rows), about 8 units of 16 bytes per thread
+  // as for greedy acceptance: few sequences, about 8 units of 16 bytes per
+  // thread
   if (static_cast<long long>(Bt) * kSampMaxCluster > num_sms) return 0;
   const long long rows = 2LL * gamma + 1;
   // at least 3 MiB of logits a sequence (measured with the current second

@@ -5,14 +5,16 @@
 // query rows that share a KV head are packed 8 to a warp, up to eight warps a
 // row block, so every K/V row is read once for all of them (one CTA per query
 // row re-read the whole cache 16 to 256 times through L2: 8 sequences of 512
-// to 1024 keys, 16/8 heads, 4 drafts, d 128 took 176 us against 26.8 us here;
-// 8 of 1024 to 2048 keys, 32/8 heads, 16 drafts 1809 against 262; one of 4096
-// keys 241 against 42.7; 50.6 MB at 26.8 us is 1.9 TB/s, bound by latency and
-// instruction issue at ten warps an SM, the large one by issue at 24 TFLOP/s).
-// Keys come in tiles
-// of 32: the paged prefix rows, then the new slots admitted by Eq. (1).  A
-// producer warp fetches them, lane i key i's row with one bulk copy, into rows
-// padded against bank conflicts.
+// to 1024 keys, 16/8 heads, 4 drafts, d 128 took 149 us against 23.0 us here;
+// 8 of 1024 to 2048 keys, 32/8 heads, 16 drafts 1789 against 255; one of 4096
+// keys, 16/8 heads, 4 drafts 155 against 38.1).  What bounds it, by counters:
+// the first (2.2 TB/s, 13 warps an SM) issues in 33% of the cycles, its warps
+// waiting for one another at the cluster barriers (ranges of unequal length),
+// for fixed latencies and for K and V; the second (25 TFLOP/s, nine warps on
+// each of 128 SMs) issues in 43% with the FMA pipe 54% busy and waits for
+// shared-memory loads.  Keys come in tiles of 32: the paged prefix rows, then
+// the new slots admitted by Eq. (1).  A producer warp fetches them, lane i key
+// i's row with one bulk copy, into rows padded against bank conflicts.
 //   S = Q K^T  a lane owns two keys (k, k + 16) and four of the warp's rows
 //              (the half-warps take the even and the odd ones): per 4
 //              elements of d two 16-byte loads of K and four broadcast loads

@@ -429,8 +429,7 @@ __global__ void __maxnreg__(kMaxRegs)
         // then acted on at once (a tile's chain of S, softmax and PV is serial
         // within a CTA, 1.2 us of which the tensor core works 0.3; waiting in
         // this order and issuing the next S ahead of the commits: 64
-        // sequences of 2048 to 8192 keys 213.7 -> 205.6 us, 32 x 4096 93.4 ->
-        // 86.1, 36 layers of 8 short sequences 824 -> 768)
+        // sequences of 2048 to 8192 keys, 16 drafts 213.9 -> 204.2 us)
         if (!mbar_wait(smem_u32(&sm.bar_v[st]), par, abort_flag, p.wait_ns) ||
             !mbar_wait(smem_u32(&sm.bar_p), i & 1, abort_flag, p.wait_ns)) {
           ok = false;
@@ -657,8 +656,8 @@ __global__ void __maxnreg__(kMaxRegs)
     if (!ok && lane == 0) signal_abort(sm, p.err_word);
     // the next kernel on the stream may be scheduled now (its CTAs wait for
     // this grid to finish anyway); a clustered grid too, ahead of its merge:
-    // the next layer's set-up then runs under it (36 layers of 8 sequences,
-    // 809 us with the trigger at exit, 768 here)
+    // the next layer's set-up then runs under it (36 layers of 8 sequences of
+    // 512 to 2048 keys, 16 drafts: 734 us with the trigger at exit, 703 here)
     pdl_launch_next();
     // ---- epilogue: O of the last PV, scaled by 1/l (bar_pv has one phase: it
     // completes when every MMA of the CTA has)
@@ -1014,7 +1013,7 @@ bool plan_attention_tc(int Bt, int gamma, int Hq, int Hkv, int max_pages, int pa
 // small batch), a warp per row otherwise (a large grid merging a few splits a
 // row needs its blocks resident more than loads in flight).  The whole call at
 // one sequence, 38 splits of each row, a warp a row -> a block a row: 32768
-// keys 35.4 -> 32.6 us, 8192 keys 18.4 -> 15.2.
+// keys 35.4 -> 32.6 us, 8192 keys 18.4 -> 15.2 (31.7 and 13.7 by now).
 cudaError_t launch_combine(const TcParams& p, long long rows, int num_sms, cudaStream_t stream) {
   if (p.nsplit > 4 && p.nsplit <= 4 * kRowPer && rows <= 16LL * num_sms)
     return launch_overlapped(combine_row_kernel, dim3(static_cast<unsigned>(rows)), dim3(128), 0, stream, 1, p);

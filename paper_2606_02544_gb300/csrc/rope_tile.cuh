@@ -7,12 +7,13 @@
 // of one slot (16 threads a slot), forms their sines and cosines once and
 // turns that slot's g query rows and its new key with them.  One query row a
 // thread, each forming all 64 pairs' angles, was bound by the sine and cosine
-// instructions.  Measured, a call without -> with rotation, row layout and
-// this one: 8 sequences of 512 to 2048 keys, 8 drafts, 32/8 heads 20.8 ->
-// 39.6 and 22.4 us; 19 of 190 to 3000 keys, 7 drafts 41.6 -> 79.1 and 43.1;
-// 32 x 4096 keys 93.9 -> 137.5 and 96.0; 32 drafts, 32 sequences of 2048 to
-// 8192 keys (the 256-row kernel, once per piece of a unit) 190 -> 240 and
-// 225.
+// instructions.  Measured, a call without -> with rotation, in the kernels
+// that had the row layout and in today's (which are faster without it, too),
+// 32/8 heads: 8 sequences of 512 to 2048 keys, 8 drafts (64 rows) 20.1 -> 38.8
+// and 14.8 -> 17.9 us, 16 drafts (128 rows) 22.6 -> 42.3 and 19.3 -> 22.3; 19
+// of 190 to 3000 keys, 7 drafts 41.7 -> 80.2 and 32.0 -> 34.1; 32 x 4096 keys,
+// 16 drafts 95.3 -> 139.5 and 87.5 -> 91.9; 32 drafts, 32 sequences of 2048 to
+// 8192 keys (256 rows, once per piece of a unit) 188 -> 240 and 173 -> 194.
 #pragma once
 #include "common.cuh"
 #include "kernels.h"
